@@ -209,6 +209,7 @@ struct fcm_handle {
   PairConsts<float> pf{};
   PairConsts<double> pd{};
   PairTable ptab{};
+  PairTable64 ptab64{};
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   BinBuffers bb{};
@@ -436,7 +437,7 @@ int launch_pair_stage(fcm_handle* h, const Geometry<R>& g, const BinBuffers& bb,
   FCM_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   if ((rc = stage_begin(h, 4, h->side, &t_pair))) return rc;
   if constexpr (std::is_same<R, double>::value)
-    launch_pair_f64(g, h->pd, torque, bb, n, up, wp, h->side, &h->launches);
+    launch_pair_f64(g, h->pd, h->ptab64, torque, bb, n, up, wp, h->side, &h->launches);
   else
     launch_pair_f32(g, h->pf, h->ptab, torque, bb, n, up, wp, h->side, &h->launches);
   if ((rc = stage_end(h, t_pair, h->side))) return rc;
@@ -672,7 +673,15 @@ size_t workspace_estimate(const fcm_params& p, int max_systems) {
   const size_t ncplx = (size_t)(p.M[0] / 2 + 1) * p.M[1] * p.M[2];
   const size_t ntiles = (size_t)g.tiles_per * gsys, ncells = (size_t)g.cells_per * gsys;
   size_t b = 16 * n + 8 * (2 * ntiles + 1) + 8 * (ncells + 1) + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + 9 * rsz * n;
-  b += (3 * rsz * mtot + 6 * rsz * ncplx) * gsys + sizeof(float4) * 5 * kPairTableIntervals;
+  size_t table = sizeof(float4) * 5 * kPairTableIntervals;
+  if (fp64) {
+    const double r_lo = 0.5 * p.a / std::sqrt(kPi);   // (r_c may be anything where no pairs act: bounded by the box)
+    const double r_c = std::isfinite(p.r_c) ? std::min(p.r_c, std::max(p.L[0], std::max(p.L[1], p.L[2]))) : 0.0;
+    int base = 0, nint = 0;
+    pair_table64_range(r_lo * r_lo, r_c * r_c, &base, &nint);
+    table = sizeof(double) * 5 * (kPair64Degree + 1) * (size_t)nint;
+  }
+  b += (3 * rsz * mtot + 6 * rsz * ncplx) * gsys + table;
   int dims[3] = {p.M[2], p.M[1], p.M[0]};
   size_t w1 = 0, w2 = 0;
   if (cufftEstimateMany(3, dims, nullptr, 1, (int)mtot, nullptr, 1, (int)ncplx, fp64 ? CUFFT_D2Z : CUFFT_R2C,
@@ -1185,8 +1194,19 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
   A(&h->spec, h->spec_bytes * gsys);
   void* table = nullptr;
   if (!h->fp64 && pairs_on) A(&table, sizeof(float4) * 5 * kPairTableIntervals);
+  if (h->fp64 && pairs_on) {
+    pair_table64_range(h->pd.rs2, h->pd.rc2, &h->ptab64.base, &h->ptab64.n);
+    A(&table, sizeof(double) * 5 * (kPair64Degree + 1) * (size_t)h->ptab64.n);
+  }
   if (rc != FCM_OK) { std::string e = g_error; release(h); return fail(rc, e); }
-  if (table) {
+  if (h->fp64 && table) {
+    h->ptab64.coef = (const double*)table;
+    launch_pair_table64(h->pd, h->ptab64, (double*)table, nullptr);
+    if (cudaGetLastError() != cudaSuccess) {
+      release(h);
+      return fail(FCM_ERR_CUDA, "launch of the pair table kernel failed");
+    }
+  } else if (table) {
     const int nint = pair_table_intervals(0.5 * sg, std::max(p->r_c, 0.5 * sg + 1e-3), sg);
     std::vector<float4> host(5 * (size_t)nint);
     const double r_lo = 0.5 * sg;

@@ -249,6 +249,18 @@ __device__ inline void pair_coeffs_table(float r2, const PairConsts<float>& C, c
   dl = cubic(__ldg(c + 4), u);
 }
 
+// FP64 table (pair_f64.cu): polynomials of degree kPair64Degree in s = r^2 about each interval's midpoint;
+// the intervals split every octave of s into 2^kPair64Bits. Interval base + k has its index in the top
+// bits of s's exponent and mantissa; coef[(5 k + f) (degree + 1) + m] multiplies (s - mid)^m.
+constexpr int kPair64Degree = 5;
+constexpr int kPair64Bits = 7;
+struct PairTable64 {
+  const double* coef;
+  int base, n;
+};
+void pair_table64_range(double rs2, double rc2, int* base, int* n);
+void launch_pair_table64(const PairConsts<double>& pc, const PairTable64& tab, double* coef, cudaStream_t s);
+
 // Host-side construction of the constants (double), then narrowing.
 void make_pair_consts(double a, double eta, double Sigma, double Sigma_D, double r_c,
                       double r_series, PairConsts<double>* out);
@@ -363,13 +375,13 @@ void launch_pair_f32(const Geometry<float>& g, const PairConsts<float>& pc, cons
                      const BinBuffers& b, int n, float* upair, float* wpair, cudaStream_t s,
                      long long* launches);
 
-// FP64 plain path (block per particle, global FP64 atomics; thread per particle pairs).
+// FP64 path (block per particle with global FP64 atomics; half-shell pairs, pair_f64.cu).
 void launch_spread_f64(const Geometry<double>& g, const KernelConsts<double>& kc, bool torque,
                        const BinBuffers& b, int n, double* grid, cudaStream_t s, long long* launches);
 void launch_gather_f64(const Geometry<double>& g, const KernelConsts<double>& kc, bool torque,
                        const BinBuffers& b, int n, const double* grid, const double* upair,
                        const double* wpair, double* U, double* W, cudaStream_t s, long long* launches);
-void launch_pair_f64(const Geometry<double>& g, const PairConsts<double>& pc, bool torque,
+void launch_pair_f64(const Geometry<double>& g, const PairConsts<double>& pc, const PairTable64& tab, bool torque,
                      const BinBuffers& b, int n, double* upair, double* wpair, cudaStream_t s,
                      long long* launches);
 

@@ -3,10 +3,8 @@
 // * spread: one block per particle; the 3 M_G one-dimensional kernel factors
 //   sit in shared memory and each thread adds a row of M_G points to the grid
 //   with global FP64 atomics (the block-per-particle scheme of Appendix C);
-// * gather: one block per particle, thread partial sums then a block reduction;
-// * pair correction: one thread per particle over the 27 neighbour cells with
-//   the closed form in FP64 (Taylor series below r_series).
-// Formulas as in grid_f32.cu and pair_f32.cu.
+// * gather: one block per particle, thread partial sums then a block reduction.
+// Formulas as in spread_f32.cu and gather_f32.cu; the pair correction is in pair_f64.cu.
 #include "fcm_internal.cuh"
 
 namespace fcm {
@@ -139,71 +137,6 @@ __global__ void __launch_bounds__(kBpp) gather_bpp_f64(Geometry<double> g, Kerne
   }
 }
 
-__device__ inline double min_image64(double d, double L) {
-  if (d > 0.5 * L) d -= L;
-  else if (d < -0.5 * L) d += L;
-  return d;
-}
-
-template <bool TORQUE>
-__global__ void __launch_bounds__(128) pair_thread_f64(Geometry<double> g, PairConsts<double> pc, int n,
-                                                       const Vec4<double>* __restrict__ cpos,
-                                                       const Vec4<double>* __restrict__ cF,
-                                                       const Vec4<double>* __restrict__ cT,
-                                                       const int* __restrict__ cstart,
-                                                       double* __restrict__ Uo, double* __restrict__ Wo) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const Vec4<double> yi = cpos[i];
-  const int cx = cell_coord(yi.x, g.cellw_inv[0], g.mcell[0]);
-  const int cy = cell_coord(yi.y, g.cellw_inv[1], g.mcell[1]);
-  const int cz = cell_coord(yi.z, g.cellw_inv[2], g.mcell[2]);
-  double u[3] = {0, 0, 0}, w[3] = {0, 0, 0};
-  for (int ddz = -1; ddz <= 1; ++ddz)
-    for (int ddy = -1; ddy <= 1; ++ddy)
-      for (int ddx = -1; ddx <= 1; ++ddx) {
-        const int c = pmod(cx + ddx, g.mcell[0]) +
-                      g.mcell[0] * (pmod(cy + ddy, g.mcell[1]) + g.mcell[1] * pmod(cz + ddz, g.mcell[2]));
-        for (int j = cstart[c]; j < cstart[c + 1]; ++j) {
-          if (j == i) continue;
-          const Vec4<double> yj = cpos[j];
-          const double dx = min_image64(yi.x - yj.x, g.L[0]);
-          const double dy = min_image64(yi.y - yj.y, g.L[1]);
-          const double dz = min_image64(yi.z - yj.z, g.L[2]);
-          const double r2 = dx * dx + dy * dy + dz * dz;
-          if (!(r2 < pc.rc2)) continue;
-          double al, bt, cr, gm, dl;
-          pair_coeffs<double>(r2, pc, al, bt, cr, gm, dl);
-          const Vec4<double> Fj = cF[j];
-          const double xF = dx * Fj.x + dy * Fj.y + dz * Fj.z;
-          u[0] += al * Fj.x + bt * xF * dx;
-          u[1] += al * Fj.y + bt * xF * dy;
-          u[2] += al * Fj.z + bt * xF * dz;
-          if (TORQUE) {
-            const Vec4<double> Tj = cT[j];
-            u[0] += cr * (Tj.y * dz - Tj.z * dy);
-            u[1] += cr * (Tj.z * dx - Tj.x * dz);
-            u[2] += cr * (Tj.x * dy - Tj.y * dx);
-            const double xT = dx * Tj.x + dy * Tj.y + dz * Tj.z;
-            w[0] += cr * (Fj.y * dz - Fj.z * dy) + gm * Tj.x + dl * xT * dx;
-            w[1] += cr * (Fj.z * dx - Fj.x * dz) + gm * Tj.y + dl * xT * dy;
-            w[2] += cr * (Fj.x * dy - Fj.y * dx) + gm * Tj.z + dl * xT * dz;
-          }
-        }
-      }
-  const Vec4<double> Fi = cF[i];
-  const size_t o = 3 * (size_t)index_from_w(yi.w);
-  Uo[o + 0] = u[0] + pc.selfVF * Fi.x;
-  Uo[o + 1] = u[1] + pc.selfVF * Fi.y;
-  Uo[o + 2] = u[2] + pc.selfVF * Fi.z;
-  if (TORQUE && Wo) {
-    const Vec4<double> Ti = cT[i];
-    Wo[o + 0] = w[0] + pc.selfWT * Ti.x;
-    Wo[o + 1] = w[1] + pc.selfWT * Ti.y;
-    Wo[o + 2] = w[2] + pc.selfWT * Ti.z;
-  }
-}
-
 void launch_spread_f64(const Geometry<double>& g, const KernelConsts<double>& kc, bool torque,
                        const BinBuffers& b, int n, double* grid, cudaStream_t s, long long* launches) {
   if (n <= 0) return;
@@ -224,21 +157,6 @@ void launch_gather_f64(const Geometry<double>& g, const KernelConsts<double>& kc
     gather_bpp_f64<true><<<n, kBpp, 0, s>>>(g, kc, n, (const Vec4<double>*)b.t_pos, grid, up, wp, U, W);
   else
     gather_bpp_f64<false><<<n, kBpp, 0, s>>>(g, kc, n, (const Vec4<double>*)b.t_pos, grid, up, wp, U, W);
-  *launches += 1;
-}
-
-void launch_pair_f64(const Geometry<double>& g, const PairConsts<double>& pc, bool torque, const BinBuffers& b,
-                     int n, double* upair, double* wpair, cudaStream_t s, long long* launches) {
-  if (n <= 0) return;
-  const int blocks = (n + 127) / 128;
-  if (torque)
-    pair_thread_f64<true><<<blocks, 128, 0, s>>>(g, pc, n, (const Vec4<double>*)b.c_pos,
-                                                 (const Vec4<double>*)b.c_F, (const Vec4<double>*)b.c_T,
-                                                 b.cell_start, upair, wpair);
-  else
-    pair_thread_f64<false><<<blocks, 128, 0, s>>>(g, pc, n, (const Vec4<double>*)b.c_pos,
-                                                  (const Vec4<double>*)b.c_F, (const Vec4<double>*)b.c_T,
-                                                  b.cell_start, upair, wpair);
   *launches += 1;
 }
 
