@@ -40,3 +40,18 @@ def test_pair_f64_separation(r):
     Uo, Wo = s.oracle(fcm.FCM_FP64, stages=2)
     assert_parity(U, Uo, FP64_TOL, f"U r={r}")
     assert_parity(W, Wo, FP64_TOL, f"W r={r}")
+
+
+@pytest.mark.parametrize("M_G", [1, 2, 7, 10, 14, 16, 17, 24])
+@pytest.mark.parametrize("mode", ["forces", "one_width", "two_widths"])
+def test_grid_f64(M_G, mode):
+    """Spread and gather over the supports: rows that fill one round of threads, several, or part of a warp; the
+    kernel with one Gaussian, with the torque's folded in, and with the torque's own width; windows that wrap."""
+    fcm = ensure_built()
+    s = System(40, (20.0, 24.0, 16.0), (32, 27, 24), 1.4, M_G, 6.0, 17, torques=mode != "forces",
+               Sigma_D=1.7 if mode == "two_widths" else 0.0)
+    U, W = run_gpu(s, fcm.FCM_FP64, stages=1, want_W=mode != "forces")
+    Uo, Wo = s.oracle(fcm.FCM_FP64, stages=1)
+    assert_parity(U, Uo, FP64_TOL, f"U M_G={M_G} {mode}")
+    if mode != "forces":
+        assert_parity(W, Wo, FP64_TOL, f"W M_G={M_G} {mode}")
