@@ -6,11 +6,10 @@
 // tile-sorted arrays used by spread/gather and the cell-sorted arrays with
 // start offsets used by the pair correction. The rank of a particle inside its
 // bin is the value its atomic increment returned, so three kernels suffice:
-// key+count, scan, scatter. The scan leaves the counters at zero for the next call.
-// Inside a tile, particles whose window starts in the first half of the tile's x
-// range come first: they count on tile_count[t], the others on tile_count[ntiles + t]
-// and are placed from tile_start[ntiles + 1 + t] (the pencil spread steps half a
-// tile at a time along x).
+// key+count, scan, scatter. The scatter leaves the counters at zero for the next call.
+// Inside an 8-point tile particles are ordered by the quarter of the tile's x range their
+// window starts in (four counters per tile, one scan over them all): the pencil spreads
+// step along x in parts of a tile.
 #include "fcm_internal.cuh"
 
 namespace fcm {
@@ -28,29 +27,34 @@ __device__ inline int system_of(const BinBuffers& b, int i) {
 
 template <typename R>
 __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, const R* __restrict__ pos,
-                                                        BinBuffers b, int need_cells) {
+                                                        BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (b.n_dev) n = min(n, *b.n_dev);
   if (i >= n) return;
   const int sys = system_of(b, i);
   int bad = 0;
-  int t[3], c[3], xoff = 0;
+  R y[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    R y = wrap_coord(pos[3 * (size_t)i + d], g.L[d], &bad);
-    int i0 = pmod(window_start_d(g, d, y), g.M[d]);
-    t[d] = i0 / g.tile[d];
-    if (d == 0) xoff = i0 - t[0] * g.tile[0];
-    c[d] = cell_coord(y, g.cellw_inv[d], g.mcell[d]);
-  }
+  for (int d = 0; d < 3; ++d) y[d] = wrap_coord(pos[3 * (size_t)i + d], g.L[d], &bad);
   if (bad) atomicOr(b.status, kStatusNonFinite);
-  unsigned tk = (unsigned)(t[0] + g.ntile[0] * (t[1] + g.ntile[1] * t[2]));
-  if (sys) tk += (unsigned)sys * (unsigned)g.tiles_per;
-  b.tile_key[i] = tk;
-  const unsigned half = (g.tile[0] >= 2 && xoff >= (g.tile[0] >> 1)) ? 1u : 0u;
-  const unsigned rank = (unsigned)atomicAdd(&b.tile_count[tk + (half ? (unsigned)b.ntiles : 0u)], 1);
-  b.tile_rank[i] = rank | (half << 31);
-  if (need_cells) {
+  if (need & kBinTiles) {
+    int t[3], xoff = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int i0 = pmod(window_start_d(g, d, y[d]), g.M[d]);
+      t[d] = i0 / g.tile[d];
+      if (d == 0) xoff = i0 - t[0] * g.tile[0];
+    }
+    unsigned tk = (unsigned)(t[0] + g.ntile[0] * (t[1] + g.ntile[1] * t[2]));
+    if (sys) tk += (unsigned)sys * (unsigned)g.tiles_per;
+    tk = kTileParts * tk + (g.tile[0] == 2 * kTileParts ? (unsigned)(xoff >> 1) : 0u);
+    b.tile_key[i] = tk;
+    b.tile_rank[i] = (unsigned)atomicAdd(&b.tile_count[tk], 1);
+  }
+  if (need & kBinCells) {
+    int c[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) c[d] = cell_coord(y[d], g.cellw_inv[d], g.mcell[d]);
     unsigned ck = (unsigned)(c[0] + g.mcell[0] * (c[1] + g.mcell[1] * c[2]));
     if (sys) ck += (unsigned)sys * (unsigned)g.cells_per;
     b.cell_key[i] = ck;
@@ -58,78 +62,119 @@ __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, co
   }
 }
 
-// Exclusive scan of one counter array by one block, offset by base; start[nb] = base + total
-// when write_end. Resets counts. With count1 (a second counter per bin, placed after the first's
-// particles), bin k holds count[k] + count1[k] particles and start1[k] = start[k] + count[k].
-__device__ void block_scan(int* count, int* start, int nb, int base, bool write_end, int* count1 = nullptr,
-                           int* start1 = nullptr) {
-  __shared__ int warp_sums[32];
-  __shared__ int carry;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int chunk = (nb + nthr - 1) / nthr;
-  const int lo = min(nb, tid * chunk), hi = min(nb, lo + chunk);
-  int local = 0;
-  for (int k = lo; k < hi; ++k) local += count[k] + (count1 ? count1[k] : 0);
-  // inclusive warp scan of the per-thread sums
-  int lane = tid & 31, wid = tid >> 5;
-  int v = local;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int u = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += u;
-  }
-  if (lane == 31) warp_sums[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    int nw = (nthr + 31) / 32;
-    int w = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int u = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += u;
-    }
-    if (lane < nw) warp_sums[lane] = w;
-    if (lane == nw - 1) carry = w;
-  }
-  __syncthreads();
-  int excl = base + v - local + (wid > 0 ? warp_sums[wid - 1] : 0);
-  for (int k = lo; k < hi; ++k) {
-    const int cnt = count[k];
-    start[k] = excl;
-    excl += cnt;
-    count[k] = 0;
-    if (count1) {
-      start1[k] = excl;
-      excl += count1[k];
-      count1[k] = 0;
-    }
-  }
-  if (tid == 0 && write_end) start[nb] = base + carry;
+// Counters of one system's bins: [first, first + nb) of count, split into chunks of kScanChunk.
+struct ScanPart {
+  const int* count;
+  int nb, chunk;
+  bool tiles, last;   // tile counters (kTileParts per tile); the launch's last system
+};
+
+__device__ inline ScanPart scan_part(const BinBuffers& b, int tile_chunks) {
+  const int sys = blockIdx.y, nsys = max(b.nsys, 1);
+  ScanPart p;
+  p.tiles = (int)blockIdx.x < tile_chunks;
+  p.nb = (p.tiles ? kTileParts * b.ntiles : b.ncells) / nsys;
+  p.chunk = p.tiles ? blockIdx.x : blockIdx.x - tile_chunks;
+  p.count = (p.tiles ? b.tile_count : b.cell_count) + (size_t)sys * p.nb;
+  p.last = sys == nsys - 1;
+  return p;
 }
 
-// Block (k, s): k = 0 scans system s's tile counters, k = 1 its cell counters. A system's
-// bins are contiguous and its particles are the stacked rows from sys_off[s], so each
-// segment starts at sys_off[s] and the segments scan independently.
-__global__ void __launch_bounds__(1024) scan_kernel(BinBuffers b, int need_cells) {
-  const int sys = blockIdx.y;
-  const int nsys = max(b.nsys, 1);
-  const int base = (b.nsys > 1 && b.sys_off) ? b.sys_off[sys] : 0;
-  const bool last = sys == nsys - 1;
-  if (blockIdx.x == 0) {
-    const int per = b.ntiles / nsys;
-    block_scan(b.tile_count + (size_t)sys * per, b.tile_start + (size_t)sys * per, per, base, last,
-               b.tile_count + (size_t)b.ntiles + (size_t)sys * per, b.tile_start + (size_t)b.ntiles + 1 + (size_t)sys * per);
-  } else if (need_cells) {
-    const int per = b.ncells / nsys;
-    block_scan(b.cell_count + (size_t)sys * per, b.cell_start + (size_t)sys * per, per, base, last);
+__device__ inline int warp_total(int v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sum of every chunk of counters (only launched for many chunks).
+__global__ void __launch_bounds__(kScanThreads) chunk_sum_kernel(BinBuffers b, int tile_chunks) {
+  __shared__ int part[kScanThreads / 32];
+  const ScanPart p = scan_part(b, tile_chunks);
+  const int lo = p.chunk * kScanChunk, hi = min(p.nb, lo + kScanChunk);
+  int v = 0;
+  for (int k = lo + threadIdx.x; k < hi; k += kScanThreads) v += p.count[k];
+  v = warp_total(v);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = warp_total(threadIdx.x < kScanThreads / 32 ? part[threadIdx.x] : 0);
+    if (threadIdx.x == 0) b.chunk_sum[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+// Exclusive scan: block (c, s) writes the starts of chunk c of system s's bins. It adds up the counters
+// before its chunk by itself (from the chunk sums when they were made), so the blocks need no order. A system's
+// bins are contiguous and its particles are the stacked rows from sys_off[s]: segments start there.
+__global__ void __launch_bounds__(kScanThreads) scan_kernel(BinBuffers b, int tile_chunks, int use_sums) {
+  __shared__ int before_w[kScanThreads / 32], own_w[kScanThreads / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const ScanPart p = scan_part(b, tile_chunks);
+  const int lo = p.chunk * kScanChunk;
+  int before = 0;
+  if (use_sums) {
+    const int* cs = b.chunk_sum + (size_t)blockIdx.y * gridDim.x + (p.tiles ? 0 : tile_chunks);
+    for (int k = threadIdx.x; k < p.chunk; k += kScanThreads) before += cs[k];
+  } else {
+#pragma unroll 8
+    for (int k = threadIdx.x; k < lo; k += kScanThreads) before += p.count[k];
+  }
+  constexpr int kPer = kScanChunk / kScanThreads;
+  const int first = lo + kPer * threadIdx.x;
+  int v[kPer], own = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    v[k] = first + k < p.nb ? p.count[first + k] : 0;
+    own += v[k];
+  }
+  before = warp_total(before);
+  int incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) {
+    before_w[wid] = before;
+    own_w[wid] = incl;
+  }
+  __syncthreads();
+  int excl = incl - own;
+  for (int w = 0; w < kScanThreads / 32; ++w) excl += before_w[w] + (w < wid ? own_w[w] : 0);
+  if (b.nsys > 1 && b.sys_off) excl += b.sys_off[blockIdx.y];
+  const size_t at = (size_t)blockIdx.y * p.nb + first;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    if (first + k < p.nb) {
+      if (p.tiles) {
+        b.part_start[at + k] = excl;
+        if ((first + k) % kTileParts == 0) b.tile_start[(at + k) / kTileParts] = excl;
+      } else {
+        b.cell_start[at + k] = excl;
+      }
+      excl += v[k];
+      if (p.last && first + k == p.nb - 1) {   // the end of the last bin
+        if (p.tiles) {
+          b.part_start[at + k + 1] = excl;
+          b.tile_start[b.ntiles] = excl;
+        } else {
+          b.cell_start[at + k + 1] = excl;
+        }
+      }
+    }
   }
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, const R* __restrict__ pos,
                                                       const R* __restrict__ F, const R* __restrict__ T,
-                                                      BinBuffers b, int need_cells) {
+                                                      BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  // the counters back to zero for the next call (16 bytes per store; the arrays are padded to 256 bytes)
+  const int nz_t = (need & kBinTiles) ? b.ntiles : 0, nz_c = (need & kBinCells) ? (b.ncells + 3) / 4 : 0;
+  static_assert(kTileParts == 4, "one 16-byte store per tile");
+  for (int k = i; k < nz_t + nz_c; k += gridDim.x * blockDim.x)
+    (k < nz_t ? reinterpret_cast<int4*>(b.tile_count)[k] : reinterpret_cast<int4*>(b.cell_count)[k - nz_t]) =
+        make_int4(0, 0, 0, 0);
   if (b.n_dev) n = min(n, *b.n_dev);
   if (i >= n) return;
   int bad = 0;
@@ -143,14 +188,14 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
   else   { t.x = R(0); t.y = R(0); t.z = R(0); }
   t.w = R(0);
   // keys and ranks come from key_count_kernel; both bins are in range by construction
-  const unsigned rk = b.tile_rank[i];
-  int dt = b.tile_start[(rk >> 31) ? (size_t)b.ntiles + 1 + b.tile_key[i] : (size_t)b.tile_key[i]] +
-           (int)(rk & 0x7fffffffu);
-  dt = min(max(dt, 0), n - 1);
-  ((Vec4<R>*)b.t_pos)[dt] = p;
-  ((Vec4<R>*)b.t_F)[dt] = f;
-  ((Vec4<R>*)b.t_T)[dt] = t;
-  if (need_cells) {
+  if (need & kBinTiles) {
+    int dt = b.part_start[b.tile_key[i]] + (int)b.tile_rank[i];
+    dt = min(max(dt, 0), n - 1);
+    ((Vec4<R>*)b.t_pos)[dt] = p;
+    ((Vec4<R>*)b.t_F)[dt] = f;
+    ((Vec4<R>*)b.t_T)[dt] = t;
+  }
+  if (need & kBinCells) {
     int dc = b.cell_start[b.cell_key[i]] + (int)b.cell_rank[i];
     dc = min(max(dc, 0), n - 1);
     ((Vec4<R>*)b.c_pos)[dc] = p;
@@ -161,19 +206,33 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
 
 template <typename R>
 void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const R* T,
-                    const BinBuffers& b, bool need_cells, cudaStream_t s, long long* launches) {
+                    const BinBuffers& b, int need, cudaStream_t s, long long* launches) {
   if (n <= 0) return;
-  int blocks = (n + 255) / 256;
-  key_count_kernel<R><<<blocks, 256, 0, s>>>(g, n, pos, b, need_cells ? 1 : 0);
-  scan_kernel<<<dim3(2, b.nsys > 1 ? b.nsys : 1), 1024, 0, s>>>(b, need_cells ? 1 : 0);
-  scatter_kernel<R><<<blocks, 256, 0, s>>>(g, n, pos, F, T, b, need_cells ? 1 : 0);
-  *launches += 3;
+  const int nsys = b.nsys > 1 ? b.nsys : 1;
+  const int tiles = (need & kBinTiles) ? b.ntiles : 0, cells = (need & kBinCells) ? b.ncells : 0;
+  const int tile_chunks = scan_chunks(kTileParts * (tiles / nsys)), cell_chunks = scan_chunks(cells / nsys);
+  const int blocks = (n + 255) / 256;
+  key_count_kernel<R><<<blocks, 256, 0, s>>>(g, n, pos, b, need);
+  *launches += 1;
+  // Every block reading all counters before its chunk costs chunks^2 / 2 chunk reads from L2: below a microsecond
+  // at 16 chunks, 8 at 64 (each block's own reads are a chain of loads); past that the chunk sums pay their launch.
+  const bool sums = std::max(tile_chunks, cell_chunks) > 32 && b.chunk_sum != nullptr;
+  const dim3 grid(tile_chunks + cell_chunks, nsys);
+  if (sums) {
+    chunk_sum_kernel<<<grid, kScanThreads, 0, s>>>(b, tile_chunks);
+    *launches += 1;
+  }
+  scan_kernel<<<grid, kScanThreads, 0, s>>>(b, tile_chunks, sums ? 1 : 0);
+  // enough blocks for the particles and for at most eight counter stores per thread
+  const int zero_blocks = (int)(((long long)tiles + cells / 4 + 1 + 2047) / 2048);
+  scatter_kernel<R><<<std::max(blocks, zero_blocks), 256, 0, s>>>(g, n, pos, F, T, b, need);
+  *launches += 2;
 }
 
 template void launch_binning<float>(const Geometry<float>&, int, const float*, const float*, const float*,
-                                    const BinBuffers&, bool, cudaStream_t, long long*);
+                                    const BinBuffers&, int, cudaStream_t, long long*);
 template void launch_binning<double>(const Geometry<double>&, int, const double*, const double*, const double*,
-                                     const BinBuffers&, bool, cudaStream_t, long long*);
+                                     const BinBuffers&, int, cudaStream_t, long long*);
 
 __global__ void write_offsets_kernel(SysOffsets o, int n, int* dst) {
   for (int k = threadIdx.x; k <= n; k += blockDim.x) dst[k] = o.off[k];

@@ -475,7 +475,7 @@ int run(fcm_handle* h, int nsys, int n, const R* pos, const R* F, const R* T, R*
   int rc, t_all, t_bin, t_spread, t_fft, t_gather;
   if ((rc = stage_begin(h, 5, s, &t_all))) return rc;
   if ((rc = stage_begin(h, 0, s, &t_bin))) return rc;
-  launch_binning<R>(g, n, pos, F, T, bb, pair_on, s, &h->launches);
+  launch_binning<R>(g, n, pos, F, T, bb, (grid_on ? kBinTiles : 0) | (pair_on ? kBinCells : 0), s, &h->launches);
   if ((rc = stage_end(h, t_bin, s))) return rc;
   FCM_CUDA(cudaGetLastError());
   if (grid_on) {
@@ -672,7 +672,7 @@ size_t workspace_estimate(const fcm_params& p, int max_systems) {
   const size_t mtot = (size_t)p.M[0] * p.M[1] * p.M[2];
   const size_t ncplx = (size_t)(p.M[0] / 2 + 1) * p.M[1] * p.M[2];
   const size_t ntiles = (size_t)g.tiles_per * gsys, ncells = (size_t)g.cells_per * gsys;
-  size_t b = 16 * n + 8 * (2 * ntiles + 1) + 8 * (ncells + 1) + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + 9 * rsz * n;
+  size_t b = 16 * n + 4 * ((2 * kTileParts + 1) * ntiles + 2) + 8 * (ncells + 1) + (kTileParts * ntiles + ncells) / 512 + 8 * gsys + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + 9 * rsz * n;
   size_t table = sizeof(float4) * 5 * kPairTableIntervals;
   if (fp64) {
     const double r_lo = 0.5 * p.a / std::sqrt(kPi);   // (r_c may be anything where no pairs act: bounded by the box)
@@ -774,7 +774,7 @@ int brownian_grid(fcm_handle* h, int n, const R* pos, const R* xi, double kT, R*
   bb.ntiles = g.tiles_per;
   const fcm_handle::Plan* plan = plan_for(h, 1);
   if (!plan) return fail(FCM_ERR_ARG, "no FFT plan for one system");
-  launch_binning<R>(g, n, pos, pos, nullptr, bb, false, s, &h->launches);   // tile order (forces unused)
+  launch_binning<R>(g, n, pos, pos, nullptr, bb, kBinTiles, s, &h->launches);   // tile order (forces unused)
   FCM_CUDA(cudaMemcpyAsync(h->grid, xi, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
   const double h3 = (h->p.L[0] / h->p.M[0]) * (h->p.L[1] / h->p.M[1]) * (h->p.L[2] / h->p.M[2]);
   const R factor = (R)std::sqrt(2.0 * kT / h3);
@@ -1181,7 +1181,9 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
   b.ncells = pairs_on ? (int)ncells_d : 1;
   A((void**)&b.tile_key, 4 * n); A((void**)&b.tile_rank, 4 * n);
   A((void**)&b.cell_key, 4 * n); A((void**)&b.cell_rank, 4 * n);
-  A((void**)&b.tile_count, 4 * (size_t)(2 * b.ntiles + 1)); A((void**)&b.tile_start, 4 * (size_t)(2 * b.ntiles + 1));
+  A((void**)&b.tile_count, 4 * (size_t)kTileParts * b.ntiles);
+  A((void**)&b.part_start, 4 * ((size_t)kTileParts * b.ntiles + 1)); A((void**)&b.tile_start, 4 * ((size_t)b.ntiles + 1));
+  A((void**)&b.chunk_sum, 4 * (size_t)gsys * (scan_chunks(kTileParts * (b.ntiles / gsys)) + scan_chunks(b.ncells / gsys)));
   A((void**)&b.cell_count, 4 * (size_t)(b.ncells + 1)); A((void**)&b.cell_start, 4 * (size_t)(b.ncells + 1));
   A(&b.t_pos, v4 * n); A(&b.t_F, v4 * n); A(&b.t_T, v4 * n);
   A(&b.c_pos, v4 * n); A(&b.c_F, v4 * n); A(&b.c_T, v4 * n);
@@ -1221,7 +1223,7 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
     h->ptab.inv_h = (float)(nint / (r_hi - r_lo));
     h->ptab.n = nint;
   }
-  cudaError_t ce = cudaMemset(b.tile_count, 0, 4 * (size_t)(2 * b.ntiles + 1));
+  cudaError_t ce = cudaMemset(b.tile_count, 0, 4 * (size_t)kTileParts * b.ntiles);
   if (ce == cudaSuccess) ce = cudaMemset(b.cell_count, 0, 4 * (size_t)(b.ncells + 1));
   if (ce == cudaSuccess) ce = cudaMemset(b.status, 0, 256);
   if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);

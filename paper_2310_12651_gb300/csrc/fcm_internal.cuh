@@ -269,12 +269,21 @@ void narrow_pair_consts(const PairConsts<double>& in, PairConsts<float>* out);
 void build_pair_table(const PairConsts<double>& pd, double r_lo, double r_hi, int n, float4* coef);
 
 // ---------------------------------------------------------------- launch API
+constexpr int kTileParts = 4;       // parts of an 8-point tile's x range by which its particles are ordered
+constexpr int kScanThreads = 512;
+constexpr int kScanChunk = 2048;    // counters per block of the scan
+inline int scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
+enum : int { kBinTiles = 1, kBinCells = 2 };   // which of the two orders a call needs
+
 // Binning: wraps positions, computes tile and cell keys, counts and ranks,
 // scans, then scatters pos/F/T into tile-sorted and cell-sorted Vec4 arrays
 // whose w field carries the original index.
 struct BinBuffers {
   unsigned* tile_key; unsigned* tile_rank; unsigned* cell_key; unsigned* cell_rank;
-  int* tile_count; int* tile_start; int* cell_count; int* cell_start;
+  int* tile_count;    // kTileParts counters per tile, in x order
+  int* part_start;    // first particle of every part of a tile
+  int* tile_start; int* cell_count; int* cell_start;
+  int* chunk_sum;     // scan: sums of kScanChunk counters (may be null for few chunks)
   int ntiles; int ncells;
   void* t_pos; void* t_F; void* t_T;   // tile-sorted Vec4<R>
   void* c_pos; void* c_F; void* c_T;   // cell-sorted Vec4<R>
@@ -295,7 +304,7 @@ void launch_write_offsets(const SysOffsets& o, int n, int* dst, cudaStream_t s, 
 
 template <typename R>
 void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const R* T,
-                    const BinBuffers& b, bool need_cells, cudaStream_t s, long long* launches);
+                    const BinBuffers& b, int need, cudaStream_t s, long long* launches);
 
 template <typename R>
 void launch_projection(const Geometry<R>& g, R eta, void* spectrum, cudaStream_t s, long long* launches);

@@ -39,12 +39,11 @@ constexpr size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign;
 constexpr size_t kN = FCM_NOALLOC_MAX_N;
 constexpr size_t kCells = FCM_NOALLOC_MAX_CELLS;
 constexpr size_t kKeysBytes = align_up(4 * sizeof(unsigned) * kN);
-constexpr size_t kTileCountBytes = align_up(2 * sizeof(int) * 2);
-constexpr size_t kCellCountBytes = align_up(2 * sizeof(int) * (kCells + 1));
+constexpr size_t kCellCountBytes = align_up(2 * sizeof(int) * (kCells + 4));
 constexpr size_t kSortedBytes = align_up(6 * sizeof(float4) * kN);
 constexpr size_t kTableBytes = align_up(5 * sizeof(float4) * kPairTableIntervals);
 constexpr size_t kStatusBytes = kAlign;
-constexpr size_t kScratchBytes = kKeysBytes + kTileCountBytes + kCellCountBytes + kSortedBytes + kTableBytes + kStatusBytes;
+constexpr size_t kScratchBytes = kKeysBytes + kCellCountBytes + kSortedBytes + kTableBytes + kStatusBytes;
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -147,11 +146,8 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
   b.cell_key = b.tile_rank + kN;
   b.cell_rank = b.cell_key + kN;
   q += kKeysBytes;
-  b.tile_count = (int*)q;
-  b.tile_start = b.tile_count + 2;
-  q += kTileCountBytes;
   b.cell_count = (int*)q;
-  b.cell_start = b.cell_count + (kCells + 1);
+  b.cell_start = b.cell_count + (kCells + 4);   // the counters are cleared 16 bytes at a time
   q += kCellCountBytes;
   float4* sorted = (float4*)q;
   b.t_pos = sorted;
@@ -182,12 +178,11 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
   cudaStream_t s = (cudaStream_t)stream;
   long long launches = 0;
   // counters must start at zero; the scan leaves them at zero, but a call may follow an error
-  launch_zero(b.tile_count, kTileCountBytes, s, &launches);
   launch_zero(b.cell_count, sizeof(int) * (size_t)(cells + 1), s, &launches);
   launch_zero(b.status, kStatusBytes, s, &launches);
   build_table_kernel<<<(kPairTableIntervals + 127) / 128, 128, 0, s>>>(pd, r_lo, (r_hi - r_lo) / kPairTableIntervals,
                                                                       kPairTableIntervals, table);
-  launch_binning<float>(g, n, (const float*)pos, (const float*)F, (const float*)T, b, true, s, &launches);
+  launch_binning<float>(g, n, (const float*)pos, (const float*)F, (const float*)T, b, kBinCells, s, &launches);
   const bool torque = (T != nullptr) || (W != nullptr);
   launch_pair_f32(g, pf, tab, torque, b, n, (float*)U, (float*)W, s, &launches);
   cudaError_t e = cudaGetLastError();
