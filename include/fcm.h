@@ -55,9 +55,9 @@ typedef enum fcm_status {
 
 typedef enum fcm_precision {
   FCM_FP32 = 0,  /* float I/O; tiled spread/gather, FP32 FFT; pair corrections from  */
-                 /* piecewise cubics fitted in FP64 to the closed forms, a Taylor    */
-                 /* series below sigma/2, per-particle pair sums compensated across  */
-                 /* candidate chunks                                                 */
+                 /* polynomials in 1/r times a Gaussian beyond a few particle radii   */
+                 /* and piecewise cubics closer, both fitted in FP64 to the closed     */
+                 /* forms, and a Taylor series below sigma/2                           */
   FCM_FP64 = 1   /* double I/O; the plain path: global FP64 atomics, FP64 FFT        */
 } fcm_precision;
 
@@ -411,7 +411,7 @@ int fcm_server_destroy(fcm_server* s);
  *            per dimension, must number at most FCM_NOALLOC_MAX_CELLS
  *   pos, F, T (T may be NULL), U, W (W may be NULL): as for fcm_apply, on the
  *            current CUDA device
- * It allocates nothing: all scratch (about 7.7 MB) is one fixed file-scope
+ * It allocates nothing: all scratch (about 6.4 MB) is one fixed file-scope
  * device array, held by every CUDA context that loads the library's device
  * code (normally one per GPU) until the process exits. With lazy module
  * loading the context reserves it at the first call made in it: make that

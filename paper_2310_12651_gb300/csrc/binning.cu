@@ -53,10 +53,16 @@ __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, co
   }
   if (need & kBinCells) {
     int c[3];
+    unsigned oct = 0;   // bit d: the upper half of the cell along d
 #pragma unroll
-    for (int d = 0; d < 3; ++d) c[d] = cell_coord(y[d], g.cellw_inv[d], g.mcell[d]);
+    for (int d = 0; d < 3; ++d) {
+      c[d] = cell_coord(y[d], g.cellw_inv[d], g.mcell[d]);
+      if (y[d] * g.cellw_inv[d] - R(c[d]) >= R(0.5)) oct |= 1u << d;
+    }
     unsigned ck = (unsigned)(c[0] + g.mcell[0] * (c[1] + g.mcell[1] * c[2]));
     if (sys) ck += (unsigned)sys * (unsigned)g.cells_per;
+    // octants in Gray-code order: consecutive ones share a face (0, 1, 3, 2, 6, 7, 5, 4 are steps 0 .. 7)
+    if (b.cell_parts == 8) ck = 8u * ck + ((oct >> 2) * 7u ^ ((oct >> 1 & 1u) * 3u) ^ (oct & 1u));
     b.cell_key[i] = ck;
     b.cell_rank[i] = (unsigned)atomicAdd(&b.cell_count[ck], 1);
   }
@@ -73,7 +79,7 @@ __device__ inline ScanPart scan_part(const BinBuffers& b, int tile_chunks) {
   const int sys = blockIdx.y, nsys = max(b.nsys, 1);
   ScanPart p;
   p.tiles = (int)blockIdx.x < tile_chunks;
-  p.nb = (p.tiles ? kTileParts * b.ntiles : b.ncells) / nsys;
+  p.nb = (p.tiles ? kTileParts * b.ntiles : b.cell_parts * b.ncells) / nsys;
   p.chunk = p.tiles ? blockIdx.x : blockIdx.x - tile_chunks;
   p.count = (p.tiles ? b.tile_count : b.cell_count) + (size_t)sys * p.nb;
   p.last = sys == nsys - 1;
@@ -149,7 +155,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(BinBuffers b, int ti
         b.part_start[at + k] = excl;
         if ((first + k) % kTileParts == 0) b.tile_start[(at + k) / kTileParts] = excl;
       } else {
-        b.cell_start[at + k] = excl;
+        b.cell_part_start[at + k] = excl;
+        if ((first + k) % b.cell_parts == 0) b.cell_start[(at + k) / b.cell_parts] = excl;
       }
       excl += v[k];
       if (p.last && first + k == p.nb - 1) {   // the end of the last bin
@@ -157,7 +164,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(BinBuffers b, int ti
           b.part_start[at + k + 1] = excl;
           b.tile_start[b.ntiles] = excl;
         } else {
-          b.cell_start[at + k + 1] = excl;
+          b.cell_part_start[at + k + 1] = excl;
+          b.cell_start[b.ncells] = excl;
         }
       }
     }
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
                                                       BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   // the counters back to zero for the next call (16 bytes per store; the arrays are padded to 256 bytes)
-  const int nz_t = (need & kBinTiles) ? b.ntiles : 0, nz_c = (need & kBinCells) ? (b.ncells + 3) / 4 : 0;
+  const int nz_t = (need & kBinTiles) ? b.ntiles : 0, nz_c = (need & kBinCells) ? (b.cell_parts * b.ncells + 3) / 4 : 0;
   static_assert(kTileParts == 4, "one 16-byte store per tile");
   for (int k = i; k < nz_t + nz_c; k += gridDim.x * blockDim.x)
     (k < nz_t ? reinterpret_cast<int4*>(b.tile_count)[k] : reinterpret_cast<int4*>(b.cell_count)[k - nz_t]) =
@@ -196,8 +204,14 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
     ((Vec4<R>*)b.t_T)[dt] = t;
   }
   if (need & kBinCells) {
-    int dc = b.cell_start[b.cell_key[i]] + (int)b.cell_rank[i];
+    int dc = b.cell_part_start[b.cell_key[i]] + (int)b.cell_rank[i];
     dc = min(max(dc, 0), n - 1);
+    b.cell_rank[i] = (unsigned)dc;   // from here on the particle's place in cell order
+    if (b.c_sum) {
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      ((float4*)b.c_sum)[2 * (size_t)dc] = zero;
+      ((float4*)b.c_sum)[2 * (size_t)dc + 1] = zero;
+    }
     ((Vec4<R>*)b.c_pos)[dc] = p;
     ((Vec4<R>*)b.c_F)[dc] = f;
     ((Vec4<R>*)b.c_T)[dc] = t;
@@ -209,7 +223,7 @@ void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const
                     const BinBuffers& b, int need, cudaStream_t s, long long* launches) {
   if (n <= 0) return;
   const int nsys = b.nsys > 1 ? b.nsys : 1;
-  const int tiles = (need & kBinTiles) ? b.ntiles : 0, cells = (need & kBinCells) ? b.ncells : 0;
+  const int tiles = (need & kBinTiles) ? b.ntiles : 0, cells = (need & kBinCells) ? b.cell_parts * b.ncells : 0;
   const int tile_chunks = scan_chunks(kTileParts * (tiles / nsys)), cell_chunks = scan_chunks(cells / nsys);
   const int blocks = (n + 255) / 256;
   key_count_kernel<R><<<blocks, 256, 0, s>>>(g, n, pos, b, need);
@@ -267,8 +281,6 @@ void launch_add(R* U, const R* up, R* W, const R* wp, size_t count, cudaStream_t
   *launches += 1;
 }
 
-template void launch_add<float>(float*, const float*, float*, const float*, size_t, cudaStream_t, long long*,
-                                const int*);
 template void launch_add<double>(double*, const double*, double*, const double*, size_t, cudaStream_t, long long*,
                                  const int*);
 

@@ -195,6 +195,137 @@ void build_pair_table(const PairConsts<double>& pd, double r_lo, double r_hi, in
   }
 }
 
+// The fit of PairPoly: for each coefficient f the weights w = exp(-r^2 / 4 Sigma^2) r^d / scale turn the error into
+// one relative to the self mobility of its block (bt and dl act with r^2, cr with r), and a polynomial in t (affine
+// in 1/r, Chebyshev basis) is fitted by iteratively reweighted least squares, whose weights tend to the minimax
+// solution. False unless all five errors, with the coefficients rounded to FP32, are below kPairPolyTol.
+constexpr double kPairPolyTol = 6e-9;   // 146 neighbours add up to 7e-8 of the self mobility at random
+
+static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn, double r_c, PairPoly* out) {
+  constexpr int D = kPairPolyDegree, N = 48;
+  PairConsts<double> pc = pd;
+  pc.rs2 = 0.0;
+  const double e4 = 1.0 / (4.0 * pd.Sg2);
+  const double vf = 1.0 / (6.0 * kPi * pd.eta * a), wt = 1.0 / (8.0 * kPi * pd.eta * a * a * a);
+  const double scale[5] = {vf, vf, std::sqrt(vf * wt), wt, wt};
+  const int power[5] = {0, 2, 1, 0, 2};
+  const double alpha = 2.0 / (1.0 / rn - 1.0 / r_c), beta = 1.0 - alpha / rn;
+  double T[N][D + 1], f[5][N], w[5][N];
+  for (int k = 0; k < N; ++k) {
+    const double t = std::cos(kPi * (k + 0.5) / N), r = alpha / (t - beta);
+    double c[5];
+    pair_coeffs<double>(r * r, pc, c[0], c[1], c[2], c[3], c[4]);
+    for (int q = 0; q < 5; ++q) {
+      const double u = (power[q] == 0 ? 1.0 : (power[q] == 1 ? r : r * r)) / scale[q];
+      f[q][k] = c[q] * u;
+      w[q][k] = std::exp(-r * r * e4) * u;
+    }
+    T[k][0] = 1.0;
+    T[k][1] = t;
+    for (int m = 2; m <= D; ++m) T[k][m] = 2.0 * t * T[k][m - 1] - T[k][m - 2];
+  }
+  double tm[D + 1][D + 1] = {};   // powers of t of the Chebyshev polynomials
+  tm[0][0] = 1.0;
+  tm[1][1] = 1.0;
+  for (int m = 2; m <= D; ++m)
+    for (int j = 0; j <= D; ++j) tm[m][j] = (j > 0 ? 2.0 * tm[m - 1][j - 1] : 0.0) - tm[m - 2][j];
+  for (int q = 0; q < 5; ++q) {
+    double lw[N], x[D + 1] = {};
+    for (int k = 0; k < N; ++k) lw[k] = 1.0;
+    for (int it = 0; it < 8; ++it) {
+      double A[D + 1][D + 2] = {};
+      for (int k = 0; k < N; ++k) {
+        const double ww = lw[k] * w[q][k] * w[q][k], wf = lw[k] * w[q][k] * f[q][k];
+        for (int i = 0; i <= D; ++i) {
+          for (int j = 0; j <= i; ++j) A[i][j] += ww * T[k][i] * T[k][j];
+          A[i][D + 1] += wf * T[k][i];
+        }
+      }
+      for (int i = 0; i <= D; ++i)
+        for (int j = i + 1; j <= D; ++j) A[i][j] = A[j][i];
+      for (int i = 0; i <= D; ++i) {   // elimination with row exchanges
+        int p = i;
+        for (int r = i + 1; r <= D; ++r)
+          if (std::fabs(A[r][i]) > std::fabs(A[p][i])) p = r;
+        for (int j = 0; j <= D + 1; ++j) std::swap(A[i][j], A[p][j]);
+        for (int r = i + 1; r <= D; ++r) {
+          const double m = A[i][i] != 0.0 ? A[r][i] / A[i][i] : 0.0;
+          for (int j = i; j <= D + 1; ++j) A[r][j] -= m * A[i][j];
+        }
+      }
+      for (int i = D; i >= 0; --i) {
+        double s = A[i][D + 1];
+        for (int j = i + 1; j <= D; ++j) s -= A[i][j] * x[j];
+        x[i] = A[i][i] != 0.0 ? s / A[i][i] : 0.0;
+      }
+      double worst = 0.0, err[N];
+      for (int k = 0; k < N; ++k) {
+        double s = 0.0;
+        for (int m = 0; m <= D; ++m) s += x[m] * T[k][m];
+        err[k] = std::fabs(w[q][k] * s - f[q][k]);
+        worst = std::max(worst, err[k]);
+      }
+      if (!(worst > 0.25 * kPairPolyTol)) break;   // good enough
+      for (int k = 0; k < N; ++k) lw[k] *= err[k] / worst + 1e-3;
+    }
+    for (int j = 0; j <= D; ++j) {
+      double s = 0.0;
+      for (int m = j; m <= D; ++m) s += x[m] * tm[m][j];
+      out->c[q][j] = (float)s;
+    }
+    for (int k = 0; k < N; ++k) {
+      double s = 0.0;
+      for (int j = D; j >= 0; --j) s = s * T[k][1] + (double)out->c[q][j];
+      if (!(std::fabs(w[q][k] * s - f[q][k]) < kPairPolyTol)) return false;
+    }
+  }
+  out->scale = (float)alpha;
+  out->offset = (float)beta;
+  out->expo = (float)(-e4 * 1.4426950408889634);
+  out->near2 = (float)(rn * rn);
+  out->ok = 1;
+  return true;
+}
+
+// The smallest r_near on a ladder from 3 sigma to 0.6 r_c (past it too many pairs would be near ones) whose fit holds
+// (the error falls with r_near). The last result of the thread is kept, since callers without a handle ask for the
+// same parameters call after call.
+void fit_pair_poly(const PairConsts<double>& pd, double a, double r_c, PairPoly* out) {
+  struct Last {
+    double key[6];
+    PairPoly poly;
+  };
+  thread_local Last last{};
+  const double key[6] = {a, pd.eta, pd.Sg2, pd.SD2, r_c, pd.sg2};
+  if (std::memcmp(key, last.key, sizeof(key)) == 0 && r_c > 0.0) {
+    *out = last.poly;
+    return;
+  }
+  PairPoly best;
+  std::memset(&best, 0, sizeof(best));
+  const double r0 = 3.0 * std::sqrt(pd.sg2), step = 1.12;
+  if (r_c > 0.0 && std::isfinite(r_c) && r0 <= 0.6 * r_c) {
+    const int top = (int)(std::log(0.6 * r_c / r0) / std::log(step));
+    auto fits = [&](int k) {
+      PairPoly p;
+      std::memset(&p, 0, sizeof(p));
+      if (!fit_pair_poly_from(pd, a, r0 * std::pow(step, k), r_c, &p)) return false;
+      best = p;
+      return true;
+    };
+    // r_near is close to 2.6 Sigma for Sigma / sigma = 1.3 .. 12 and cutoffs of 5 to 8.6 Sigma: down from there, or up
+    int k = std::min(top, std::max(0, (int)std::lround(std::log(2.6 * std::sqrt(pd.Sg2) / r0) / std::log(step))));
+    if (fits(k)) {
+      while (k > 0 && fits(k - 1)) --k;
+    } else {
+      while (k < top && !fits(k + 1)) ++k;
+    }
+  }
+  std::memcpy(last.key, key, sizeof(key));
+  last.poly = best;
+  *out = best;
+}
+
 }  // namespace fcm
 
 struct fcm_handle {
@@ -210,6 +341,7 @@ struct fcm_handle {
   PairConsts<double> pd{};
   PairTable ptab{};
   PairTable64 ptab64{};
+  PairPoly ppoly{};
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   BinBuffers bb{};
@@ -344,7 +476,9 @@ void fill_geometry(const fcm_params& p, const int tile[3], Geometry<R>* g, int s
     g->mcell[d] = (int)std::min(std::max(m, 3.0), 1048576.0);
     g->cellw_inv[d] = (R)(g->mcell[d] / p.L[d]);
   }
-  g->shift = (g->mcell[0] >= 4 && g->mcell[1] >= 4 && g->mcell[2] >= 4) ? 1 : 0;
+  g->shift = 1;
+  for (int d = 0; d < 3; ++d)
+    if (g->mcell[d] < 4 && p.L[d] < 3.0 * p.r_c * (1.0 + 1e-5)) g->shift = 0;
   g->MG = p.M_G;
   g->nsys = 1;
   g->tiles_per = g->ntile[0] * g->ntile[1] * g->ntile[2];
@@ -431,15 +565,17 @@ template <typename R>
 int launch_pair_stage(fcm_handle* h, const Geometry<R>& g, const BinBuffers& bb, int n, R* U, R* Wout, bool torque,
                       bool grid_on, cudaStream_t s) {
   int rc, t_pair;
-  R* up = grid_on ? (R*)h->upair : U;
-  R* wp = grid_on ? (R*)h->wpair : Wout;
+  [[maybe_unused]] R* up = grid_on ? (R*)h->upair : U;   // FP64; the FP32 kernel adds in cell order
+  [[maybe_unused]] R* wp = grid_on ? (R*)h->wpair : Wout;
   FCM_CUDA(cudaEventRecord(h->ev_fork, s));
   FCM_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
   if ((rc = stage_begin(h, 4, h->side, &t_pair))) return rc;
   if constexpr (std::is_same<R, double>::value)
     launch_pair_f64(g, h->pd, h->ptab64, torque, bb, n, up, wp, h->side, &h->launches);
-  else
-    launch_pair_f32(g, h->pf, h->ptab, torque, bb, n, up, wp, h->side, &h->launches);
+  else {
+    launch_pair_f32(g, h->pf, h->ptab, h->ppoly, torque, bb, n, h->side, &h->launches);
+    if (!grid_on) launch_pair_merge(h->pf, torque, bb, n, false, U, Wout, h->side, &h->launches);
+  }
   if ((rc = stage_end(h, t_pair, h->side))) return rc;
   FCM_CUDA(cudaGetLastError());
   FCM_CUDA(cudaEventRecord(h->ev_join, h->side));
@@ -521,7 +657,10 @@ int run(fcm_handle* h, int nsys, int n, const R* pos, const R* F, const R* T, R*
       FCM_CUDA(cudaGetLastError());
       if (pair_on) {
         FCM_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
-        launch_add<R>(U, (const R*)h->upair, Wout, (const R*)h->wpair, 3 * (size_t)n, s, &h->launches, n_dev);
+        if constexpr (std::is_same<R, double>::value)
+          launch_add<R>(U, (const R*)h->upair, Wout, (const R*)h->wpair, 3 * (size_t)n, s, &h->launches, n_dev);
+        else
+          launch_pair_merge(h->pf, torque, bb, n, true, U, Wout, s, &h->launches);
         FCM_CUDA(cudaGetLastError());
       }
     }
@@ -672,7 +811,7 @@ size_t workspace_estimate(const fcm_params& p, int max_systems) {
   const size_t mtot = (size_t)p.M[0] * p.M[1] * p.M[2];
   const size_t ncplx = (size_t)(p.M[0] / 2 + 1) * p.M[1] * p.M[2];
   const size_t ntiles = (size_t)g.tiles_per * gsys, ncells = (size_t)g.cells_per * gsys;
-  size_t b = 16 * n + 4 * ((2 * kTileParts + 1) * ntiles + 2) + 8 * (ncells + 1) + (kTileParts * ntiles + ncells) / 512 + 8 * gsys + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + 9 * rsz * n;
+  size_t b = 16 * n + 4 * ((2 * kTileParts + 1) * ntiles + 2) + 4 * ((fp64 ? 1 : 17) * ncells + 2) + 4 * (ncells + 1) + (kTileParts * ntiles + 8 * ncells) / 512 + 8 * gsys + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + (fp64 ? 9 : 11) * rsz * n;
   size_t table = sizeof(float4) * 5 * kPairTableIntervals;
   if (fp64) {
     const double r_lo = 0.5 * p.a / std::sqrt(kPi);   // (r_c may be anything where no pairs act: bounded by the box)
@@ -1183,13 +1322,22 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
   A((void**)&b.cell_key, 4 * n); A((void**)&b.cell_rank, 4 * n);
   A((void**)&b.tile_count, 4 * (size_t)kTileParts * b.ntiles);
   A((void**)&b.part_start, 4 * ((size_t)kTileParts * b.ntiles + 1)); A((void**)&b.tile_start, 4 * ((size_t)b.ntiles + 1));
-  A((void**)&b.chunk_sum, 4 * (size_t)gsys * (scan_chunks(kTileParts * (b.ntiles / gsys)) + scan_chunks(b.ncells / gsys)));
-  A((void**)&b.cell_count, 4 * (size_t)(b.ncells + 1)); A((void**)&b.cell_start, 4 * (size_t)(b.ncells + 1));
+  b.cell_parts = h->fp64 ? 1 : 8;
+  A((void**)&b.cell_count, 4 * (size_t)b.cell_parts * b.ncells); A((void**)&b.cell_start, 4 * (size_t)(b.ncells + 1));
+  if (b.cell_parts == 1) b.cell_part_start = b.cell_start;
+  else A((void**)&b.cell_part_start, 4 * ((size_t)b.cell_parts * b.ncells + 1));
+  A((void**)&b.chunk_sum, 4 * (size_t)gsys * (scan_chunks(kTileParts * (b.ntiles / gsys)) + scan_chunks(b.cell_parts * (b.ncells / gsys))));
   A(&b.t_pos, v4 * n); A(&b.t_F, v4 * n); A(&b.t_T, v4 * n);
   A(&b.c_pos, v4 * n); A(&b.c_F, v4 * n); A(&b.c_T, v4 * n);
   A((void**)&b.status, 256);
   A((void**)&h->sys_off, sizeof(int) * (kMaxBatch + 1));
-  A(&h->upair, 3 * rsz * n); A(&h->wpair, 3 * rsz * n); A(&h->wscratch, 3 * rsz * n);
+  if (h->fp64) {
+    A(&h->upair, 3 * rsz * n);
+    A(&h->wpair, 3 * rsz * n);
+  } else {
+    A(&b.c_sum, 2 * sizeof(float4) * n);
+  }
+  A(&h->wscratch, 3 * rsz * n);
   h->grid_bytes = 3 * rsz * mtot;
   h->spec_bytes = 3 * 2 * rsz * ncplx;
   A(&h->grid, h->grid_bytes * gsys);
@@ -1222,9 +1370,10 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
     h->ptab.r0 = (float)r_lo;
     h->ptab.inv_h = (float)(nint / (r_hi - r_lo));
     h->ptab.n = nint;
+    fit_pair_poly(h->pd, p->a, p->r_c, &h->ppoly);
   }
   cudaError_t ce = cudaMemset(b.tile_count, 0, 4 * (size_t)kTileParts * b.ntiles);
-  if (ce == cudaSuccess) ce = cudaMemset(b.cell_count, 0, 4 * (size_t)(b.ncells + 1));
+  if (ce == cudaSuccess) ce = cudaMemset(b.cell_count, 0, 4 * (size_t)b.cell_parts * b.ncells);
   if (ce == cudaSuccess) ce = cudaMemset(b.status, 0, 256);
   if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
   if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);

@@ -59,8 +59,8 @@ struct Geometry {
   int tile[3];   // spread/gather tile in grid points
   int ntile[3];  // ceil(M_i / tile_i)
   int mcell[3];  // pair cells per dimension, max(int(L_i / r_c), 3)
-  int shift;     // 1 if every mcell >= 4: the 27-cell neighbourhood never meets itself, so a
-                 // neighbour cell's periodic image relative to the centre cell is unique
+  int shift;     // 1 if in every dimension mcell >= 4 or a cell is at least r_c wide: a pair within r_c then lies in
+                 // one periodic image of the neighbour cell, the one beside the centre cell
   // Batched launches: nsys systems with these parameters, stacked. Tile t of the launch belongs
   // to system t / tiles_per, pair cell c to system c / cells_per, and system s's grid starts
   // grid_stride reals after system s-1's. nsys <= 1 is one system (the other fields unused).
@@ -249,6 +249,17 @@ __device__ inline void pair_coeffs_table(float r2, const PairConsts<float>& C, c
   dl = cubic(__ldg(c + 4), u);
 }
 
+// FP32 coefficients beyond r_near (pair_f32.cu): c[f] holds function f (al, bt, cr, gm, dl) as
+// exp2(r^2 expo) sum_m c[f][m] t^m with t = scale / r + offset in [-1, 1] on [r_near, r_c]; near2 = r_near^2.
+// ok == 0: no such fit, every pair uses the table.
+constexpr int kPairPolyDegree = 9;
+struct PairPoly {
+  float c[5][kPairPolyDegree + 1];
+  float scale, offset, expo, near2;
+  int ok;
+};
+void fit_pair_poly(const PairConsts<double>& pd, double a, double r_c, PairPoly* out);
+
 // FP64 table (pair_f64.cu): polynomials of degree kPair64Degree in s = r^2 about each interval's midpoint;
 // the intervals split every octave of s into 2^kPair64Bits. Interval base + k has its index in the top
 // bits of s's exponent and mantissa; coef[(5 k + f) (degree + 1) + m] multiplies (s - mid)^m.
@@ -282,11 +293,15 @@ struct BinBuffers {
   unsigned* tile_key; unsigned* tile_rank; unsigned* cell_key; unsigned* cell_rank;
   int* tile_count;    // kTileParts counters per tile, in x order
   int* part_start;    // first particle of every part of a tile
-  int* tile_start; int* cell_count; int* cell_start;
+  int* tile_start;
+  int* cell_count;    // cell_parts counters per cell: its octants along a path of neighbours (8), or the cell (1)
+  int* cell_part_start;   // first particle of every part (cell_start itself where cell_parts == 1)
+  int* cell_start; int cell_parts;
   int* chunk_sum;     // scan: sums of kScanChunk counters (may be null for few chunks)
   int ntiles; int ncells;
   void* t_pos; void* t_F; void* t_T;   // tile-sorted Vec4<R>
   void* c_pos; void* c_F; void* c_T;   // cell-sorted Vec4<R>
+  void* c_sum;   // FP32: pair sums (float4 of U, float4 of W) per cell-sorted particle, cleared by the scatter
   int* status;
   // Batched launches: particles of system s are rows sys_off[s] .. sys_off[s+1]-1 of the stacked
   // inputs (device array of nsys + 1 ints); nsys <= 1 or sys_off == nullptr is one system.
@@ -380,9 +395,11 @@ inline int device_sm_count() {
 void launch_gather_f32(const Geometry<float>& g, const KernelConsts<float>& kc, bool torque,
                        const BinBuffers& b, const float* grid, const float* upair, const float* wpair,
                        float* U, float* W, cudaStream_t s, long long* launches);
-void launch_pair_f32(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab, bool torque,
-                     const BinBuffers& b, int n, float* upair, float* wpair, cudaStream_t s,
-                     long long* launches);
+void launch_pair_f32(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab, const PairPoly& poly,
+                     bool torque, const BinBuffers& b, int n, cudaStream_t s, long long* launches);
+// Pair sums and self terms from cell order to input order: U, W = or (add) +=.
+void launch_pair_merge(const PairConsts<float>& pc, bool torque, const BinBuffers& b, int n, bool add, float* U, float* W,
+                       cudaStream_t s, long long* launches);
 
 // FP64 path (block per particle with global FP64 atomics; half-shell pairs, pair_f64.cu).
 void launch_spread_f64(const Geometry<double>& g, const KernelConsts<double>& kc, bool torque,

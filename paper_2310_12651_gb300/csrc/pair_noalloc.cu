@@ -38,9 +38,9 @@ constexpr size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign;
 
 constexpr size_t kN = FCM_NOALLOC_MAX_N;
 constexpr size_t kCells = FCM_NOALLOC_MAX_CELLS;
-constexpr size_t kKeysBytes = align_up(4 * sizeof(unsigned) * kN);
+constexpr size_t kKeysBytes = align_up(2 * sizeof(unsigned) * kN);
 constexpr size_t kCellCountBytes = align_up(2 * sizeof(int) * (kCells + 4));
-constexpr size_t kSortedBytes = align_up(6 * sizeof(float4) * kN);
+constexpr size_t kSortedBytes = align_up(5 * sizeof(float4) * kN);
 constexpr size_t kTableBytes = align_up(5 * sizeof(float4) * kPairTableIntervals);
 constexpr size_t kStatusBytes = kAlign;
 constexpr size_t kScratchBytes = kKeysBytes + kCellCountBytes + kSortedBytes + kTableBytes + kStatusBytes;
@@ -128,7 +128,9 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
     cells *= g.mcell[d];
   }
   g.MG = 1;
-  g.shift = (g.mcell[0] >= 4 && g.mcell[1] >= 4 && g.mcell[2] >= 4) ? 1 : 0;
+  g.shift = 1;
+  for (int d = 0; d < 3; ++d)
+    if (g.mcell[d] < 4 && p->L[d] < 3.0 * p->r_c * (1.0 + 1e-5)) g.shift = 0;
   if (cells > (long long)FCM_NOALLOC_MAX_CELLS)
     return fail(FCM_ERR_ARG, std::to_string(cells) + " pair cells exceed " + std::to_string(FCM_NOALLOC_MAX_CELLS) +
                                  " (the fixed scratch of the no-alloc path); r_c is too small for this box");
@@ -141,21 +143,19 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
 
   BinBuffers b{};
   unsigned char* q = base;
-  b.tile_key = (unsigned*)q;
-  b.tile_rank = b.tile_key + kN;
-  b.cell_key = b.tile_rank + kN;
+  b.cell_key = (unsigned*)q;
   b.cell_rank = b.cell_key + kN;
   q += kKeysBytes;
   b.cell_count = (int*)q;
   b.cell_start = b.cell_count + (kCells + 4);   // the counters are cleared 16 bytes at a time
+  b.cell_part_start = b.cell_start;
+  b.cell_parts = 1;
   q += kCellCountBytes;
   float4* sorted = (float4*)q;
-  b.t_pos = sorted;
-  b.t_F = sorted + kN;
-  b.t_T = sorted + 2 * kN;
-  b.c_pos = sorted + 3 * kN;
-  b.c_F = sorted + 4 * kN;
-  b.c_T = sorted + 5 * kN;
+  b.c_sum = sorted;   // two float4 per particle
+  b.c_pos = sorted + 2 * kN;
+  b.c_F = sorted + 3 * kN;
+  b.c_T = sorted + 4 * kN;
   q += kSortedBytes;
   float4* table = (float4*)q;
   q += kTableBytes;
@@ -184,7 +184,10 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
                                                                       kPairTableIntervals, table);
   launch_binning<float>(g, n, (const float*)pos, (const float*)F, (const float*)T, b, kBinCells, s, &launches);
   const bool torque = (T != nullptr) || (W != nullptr);
-  launch_pair_f32(g, pf, tab, torque, b, n, (float*)U, (float*)W, s, &launches);
+  PairPoly poly;
+  fit_pair_poly(pd, p->a, p->r_c, &poly);
+  launch_pair_f32(g, pf, tab, poly, torque, b, n, s, &launches);
+  launch_pair_merge(pf, torque, b, n, false, (float*)U, (float*)W, s, &launches);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(FCM_ERR_CUDA, std::string("launch failed: ") + cudaGetErrorString(e));
   return FCM_OK;
