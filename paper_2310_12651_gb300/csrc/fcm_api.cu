@@ -355,6 +355,10 @@ struct fcm_handle {
   struct Plan { int systems; cufftHandle r2c, c2r; };
   std::vector<Plan> plans;
   void* fft_work = nullptr;
+  // The plans transform (x, y) planes and zsolve the columns in z, or (z_tw null) whole grids with a projection
+  // kernel between them, where M_z has other prime factors than 2, 3, 5 or is too long.
+  ZPlan zplan{};
+  void* z_tw = nullptr;
   int max_systems = 1;
   int* sys_off = nullptr;       // device offsets of the current batched pass
   size_t spec_bytes = 0;        // one system's spectra
@@ -588,6 +592,26 @@ const fcm_handle::Plan* plan_for(const fcm_handle* h, int nsys) {
   return nullptr;
 }
 
+// Grid -> spectrum -> operator -> grid on stream m. factor: 0 for the Stokes operator, otherwise the amplitude of its
+// square root (Brownian noise).
+template <typename R>
+int stokes_solve(fcm_handle* h, const Geometry<R>& g, const fcm_handle::Plan* plan, R factor, cudaStream_t m) {
+  FCM_CUFFT(cufftSetStream(plan->r2c, m));
+  FCM_CUFFT(cufftSetStream(plan->c2r, m));
+  if constexpr (std::is_same<R, double>::value)
+    FCM_CUFFT(cufftExecD2Z(plan->r2c, (cufftDoubleReal*)h->grid, (cufftDoubleComplex*)h->spec));
+  else
+    FCM_CUFFT(cufftExecR2C(plan->r2c, (cufftReal*)h->grid, (cufftComplex*)h->spec));
+  if (h->z_tw) launch_zsolve<R>(g, h->zplan, (R)h->p.eta, factor, h->z_tw, h->spec, m, &h->launches);
+  else if (factor == R(0)) launch_projection<R>(g, (R)h->p.eta, h->spec, m, &h->launches);
+  else launch_projection_sqrt<R>(g, (R)h->p.eta, factor, h->spec, m, &h->launches);
+  if constexpr (std::is_same<R, double>::value)
+    FCM_CUFFT(cufftExecZ2D(plan->c2r, (cufftDoubleComplex*)h->spec, (cufftDoubleReal*)h->grid));
+  else
+    FCM_CUFFT(cufftExecC2R(plan->c2r, (cufftComplex*)h->spec, (cufftReal*)h->grid));
+  return FCM_OK;
+}
+
 // One pass over nsys stacked systems (nsys > 1 only on the FP32 path; h->sys_off then holds
 // the offsets). Plans cover a bucket of systems >= nsys: the bucket's extra grids are zeroed
 // with the others, so their transforms stay zero.
@@ -632,17 +656,7 @@ int run(fcm_handle* h, int nsys, int n, const R* pos, const R* F, const R* T, R*
       // ran mostly after the gather instead of beside the FFT.)
       cudaStream_t m = s;
       if ((rc = stage_begin(h, 2, m, &t_fft))) return rc;
-      FCM_CUFFT(cufftSetStream(plan->r2c, m));
-      FCM_CUFFT(cufftSetStream(plan->c2r, m));
-      if constexpr (std::is_same<R, double>::value) {
-        FCM_CUFFT(cufftExecD2Z(plan->r2c, (cufftDoubleReal*)h->grid, (cufftDoubleComplex*)h->spec));
-        launch_projection<double>(g, h->p.eta, h->spec, m, &h->launches);
-        FCM_CUFFT(cufftExecZ2D(plan->c2r, (cufftDoubleComplex*)h->spec, (cufftDoubleReal*)h->grid));
-      } else {
-        FCM_CUFFT(cufftExecR2C(plan->r2c, (cufftReal*)h->grid, (cufftComplex*)h->spec));
-        launch_projection<float>(g, (float)h->p.eta, h->spec, m, &h->launches);
-        FCM_CUFFT(cufftExecC2R(plan->c2r, (cufftComplex*)h->spec, (cufftReal*)h->grid));
-      }
+      if ((rc = stokes_solve<R>(h, g, plan, R(0), m))) return rc;
       if ((rc = stage_end(h, t_fft, m))) return rc;
       FCM_CUDA(cudaGetLastError());
       // the gather writes the grid part; the pair sums, which run beside the FFT and the gather,
@@ -821,14 +835,20 @@ size_t workspace_estimate(const fcm_params& p, int max_systems) {
     table = sizeof(double) * 5 * (kPair64Degree + 1) * (size_t)nint;
   }
   b += (3 * rsz * mtot + 6 * rsz * ncplx) * gsys + table;
+  ZPlan zp;
+  const bool zs = make_zplan(p.M[2], fp64, &zp) && 3LL * gsys * p.M[2] < (1LL << 31);
   int dims[3] = {p.M[2], p.M[1], p.M[0]};
+  const int rank = zs ? 2 : 3, batch = zs ? 3 * gsys * p.M[2] : 3 * gsys;
+  const int real = (int)(zs ? mtot / p.M[2] : mtot), cplx = (int)(zs ? ncplx / p.M[2] : ncplx);
+  int* dim = zs ? dims + 1 : dims;
   size_t w1 = 0, w2 = 0;
-  if (cufftEstimateMany(3, dims, nullptr, 1, (int)mtot, nullptr, 1, (int)ncplx, fp64 ? CUFFT_D2Z : CUFFT_R2C,
-                        3 * gsys, &w1) != CUFFT_SUCCESS)
+  if (cufftEstimateMany(rank, dim, nullptr, 1, real, nullptr, 1, cplx, fp64 ? CUFFT_D2Z : CUFFT_R2C, batch, &w1) !=
+      CUFFT_SUCCESS)
     w1 = 6 * rsz * ncplx * gsys;
-  if (cufftEstimateMany(3, dims, nullptr, 1, (int)ncplx, nullptr, 1, (int)mtot, fp64 ? CUFFT_Z2D : CUFFT_C2R,
-                        3 * gsys, &w2) != CUFFT_SUCCESS)
+  if (cufftEstimateMany(rank, dim, nullptr, 1, cplx, nullptr, 1, real, fp64 ? CUFFT_Z2D : CUFFT_C2R, batch, &w2) !=
+      CUFFT_SUCCESS)
     w2 = w1;
+  b += 2 * rsz * (size_t)p.M[2];
   return b + std::max(w1, w2) + 24 * 256;
 }
 
@@ -917,19 +937,11 @@ int brownian_grid(fcm_handle* h, int n, const R* pos, const R* xi, double kT, R*
   FCM_CUDA(cudaMemcpyAsync(h->grid, xi, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
   const double h3 = (h->p.L[0] / h->p.M[0]) * (h->p.L[1] / h->p.M[1]) * (h->p.L[2] / h->p.M[2]);
   const R factor = (R)std::sqrt(2.0 * kT / h3);
-  FCM_CUFFT(cufftSetStream(plan->r2c, s));
-  FCM_CUFFT(cufftSetStream(plan->c2r, s));
-  if constexpr (std::is_same<R, double>::value) {
-    FCM_CUFFT(cufftExecD2Z(plan->r2c, (cufftDoubleReal*)h->grid, (cufftDoubleComplex*)h->spec));
-    launch_projection_sqrt<double>(g, h->p.eta, factor, h->spec, s, &h->launches);
-    FCM_CUFFT(cufftExecZ2D(plan->c2r, (cufftDoubleComplex*)h->spec, (cufftDoubleReal*)h->grid));
+  if (int rc = stokes_solve<R>(h, g, plan, factor, s)) return rc;
+  if constexpr (std::is_same<R, double>::value)
     launch_gather_f64(g, h->kd, W != nullptr, bb, n, (const double*)h->grid, nullptr, nullptr, U, W, s, &h->launches);
-  } else {
-    FCM_CUFFT(cufftExecR2C(plan->r2c, (cufftReal*)h->grid, (cufftComplex*)h->spec));
-    launch_projection_sqrt<float>(g, (float)h->p.eta, factor, h->spec, s, &h->launches);
-    FCM_CUFFT(cufftExecC2R(plan->c2r, (cufftComplex*)h->spec, (cufftReal*)h->grid));
+  else
     launch_gather_f32(g, h->kf, W != nullptr, bb, (const float*)h->grid, nullptr, nullptr, U, W, s, &h->launches);
-  }
   FCM_CUDA(cudaGetLastError());
   return FCM_OK;
 }
@@ -1379,13 +1391,23 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
   if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
   if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
   if (ce != cudaSuccess) { release(h); return fail(FCM_ERR_CUDA, std::string("setup: ") + cudaGetErrorString(ce)); }
-  // One R2C and one C2R plan per bucket of systems (3 transforms per system), all with one work
+  // One R2C and one C2R plan per bucket of systems (3 components per system), all with one work
   // area of the largest size any of them needs.
   int dims[3] = {p->M[2], p->M[1], p->M[0]};
   std::vector<int> buckets;
   for (int k = 1; k < gsys; k *= 2) buckets.push_back(k);
   buckets.push_back(gsys);
   size_t work = 0;
+  const bool zs = make_zplan(p->M[2], h->fp64, &h->zplan) && 3LL * gsys * p->M[2] < (1LL << 31);
+  if (zs) {
+    const size_t tb = 2 * rsz * (size_t)p->M[2];
+    std::vector<char> tw(tb);
+    z_twiddles(p->M[2], h->fp64, tw.data());
+    A(&h->z_tw, tb);
+    if (rc == FCM_OK && cudaMemcpy(h->z_tw, tw.data(), tb, cudaMemcpyHostToDevice) != cudaSuccess)
+      rc = fail(FCM_ERR_CUDA, "copy of the twiddle factors failed");
+    if (rc != FCM_OK) { std::string e = g_error; release(h); return fail(rc, e); }
+  }
   for (int nb : buckets) {
     fcm_handle::Plan pl{nb, 0, 0};
     size_t w1 = 0, w2 = 0;
@@ -1398,12 +1420,16 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
       h->plans.push_back(pl);
       fr = cufftSetAutoAllocation(pl.r2c, 0);
       if (fr == CUFFT_SUCCESS) fr = cufftSetAutoAllocation(pl.c2r, 0);
+      // (x, y) planes of every z, or whole grids
+      const int rank = zs ? 2 : 3, batch = zs ? 3 * nb * p->M[2] : 3 * nb;
+      int* dim = zs ? dims + 1 : dims;
+      const int real = (int)(zs ? mtot / p->M[2] : mtot), cplx = (int)(zs ? ncplx / p->M[2] : ncplx);
       if (fr == CUFFT_SUCCESS)
-        fr = cufftMakePlanMany(pl.r2c, 3, dims, nullptr, 1, (int)mtot, nullptr, 1, (int)ncplx,
-                               h->fp64 ? CUFFT_D2Z : CUFFT_R2C, 3 * nb, &w1);
+        fr = cufftMakePlanMany(pl.r2c, rank, dim, nullptr, 1, real, nullptr, 1, cplx, h->fp64 ? CUFFT_D2Z : CUFFT_R2C,
+                               batch, &w1);
       if (fr == CUFFT_SUCCESS)
-        fr = cufftMakePlanMany(pl.c2r, 3, dims, nullptr, 1, (int)ncplx, nullptr, 1, (int)mtot,
-                               h->fp64 ? CUFFT_Z2D : CUFFT_C2R, 3 * nb, &w2);
+        fr = cufftMakePlanMany(pl.c2r, rank, dim, nullptr, 1, cplx, nullptr, 1, real, h->fp64 ? CUFFT_Z2D : CUFFT_C2R,
+                               batch, &w2);
     }
     if (fr != CUFFT_SUCCESS) {
       release(h);

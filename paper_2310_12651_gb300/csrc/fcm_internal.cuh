@@ -328,6 +328,20 @@ template <typename R>
 void launch_projection_sqrt(const Geometry<R>& g, R eta, R factor, void* spectrum, cudaStream_t s,
                             long long* launches);
 
+// Transform along z, operator (or, factor != 0, factor times its square root), transform back (zsolve.cu): the steps
+// of a transform of length N = 2^a 3^b 5^c.
+constexpr int kZMaxSteps = 12;
+struct ZPlan {
+  int N, steps, lines_log2;   // columns per block
+  int radix[kZMaxSteps], n[kZMaxSteps], tstep[kZMaxSteps];   // n: product of the earlier radices; tstep = N / (n radix)
+  unsigned magic[kZMaxSteps];                                // division by n
+};
+bool make_zplan(int N, bool fp64, ZPlan* p);   // false where the length is not of that form or too long
+void z_twiddles(int N, bool fp64, void* host);   // N complex values exp(-2 pi i k / N)
+template <typename R>
+void launch_zsolve(const Geometry<R>& g, const ZPlan& p, R eta, R factor, const void* table, void* spectrum,
+                   cudaStream_t s, long long* launches);
+
 // Vector kernels of the Lanczos iteration (length m, FP64 accumulation of dot products).
 constexpr int kLanczosMax = 64;
 struct LanczosCoef { double c[kLanczosMax]; };
