@@ -275,13 +275,24 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_rows_kernel(Geome
 // Particles staged per pass of the pencil kernel. The profile tables are double-buffered: while
 // the row updates of pass c read one table set, the same threads build the tables of pass c + 1 in
 // the other (a warp whose rows finish early starts on them at once), and the raw rows (position,
-// force, torque) of pass c + 2 arrive by asynchronous copies. One CTA barrier per pass. Passes of
-// 128 particles where both table sets fit shared memory (one width and M_G <= 14), else 64.
+// force, torque) of pass c + 2 arrive by asynchronous copies. One CTA barrier per pass. Passes of 64
+// particles, so that two CTAs' table sets fit shared memory; 128 where one CTA has the SM (M_G = 14).
 enum { kPencilForces = 0, kPencilSameWidth = 1, kPencilTwoWidths = 2 };
 
 __host__ __device__ constexpr int pencil_chunk(int MGT, int MODE) {
-  return (MODE != kPencilTwoWidths && MGT <= 14) ? 128 : 64;
+  return (MODE != kPencilTwoWidths && MGT == 14) ? 128 : 64;
 }
+
+// Extended rows R per thread. The one-row kernel is bound by the return path of its shared loads (L1 81% busy
+// at M_G = 14): an active warp fetches 2 NP float4 of x profiles per particle for 6 NP packed FMAs. With two
+// rows a thread fetches them once for both, in half the warps. That pays where the registers (6 EXT2 sums per
+// row) leave two CTAs per SM, M_G <= 12 with one width, and the launch fills them: 8 x 65,536 rods, M_G = 12,
+// torques 1.209 -> 1.060 ms; 65,536 spheres on 128^3 0.178 -> 0.165 ms; 122,231 on 216^3, M_G = 10, forces
+// 0.283 -> 0.247 ms. One CTA per SM with two rows is slower than one row (6 or 7 warps leave the latencies
+// bare): rods 1.364 ms; M_G = 14 with 32 x 65,536 spheres 6.00 against 5.78 ms; 2,000 spheres on 32^3 (64 CTAs)
+// 21.7 against 20.5 us. So M_G = 14 and 16, two widths and launches of one CTA per SM keep one row.
+__host__ __device__ constexpr bool pencil_two_rows(int MGT, int MODE) { return MGT <= 12 && MODE != kPencilTwoWidths; }
+constexpr int pencil_threads(int MGT, int R) { return ((rows_threads(MGT) + R - 1) / R + 31) / 32 * 32; }
 
 // Register pairs of a pencil row: the walk steps half a tile (4 points) at a time, so window pairs start at
 // pair ox / 2 with ox in [0, 4) (the binning puts each tile's particles with ox < 4 first).
@@ -295,7 +306,7 @@ struct PencilTables {
   float4* zt;   // [chunk][MGT] {g, d, B d^2, g_D} along z
   float4* pf;   // [chunk] F' = nrm F (two widths: F)
   float4* pt;   // [chunk] U' = tq T (two widths: T)
-  int4* po;     // [chunk] (x offset in the tile, y and z window start in the region, tile step)
+  int2* po;     // [chunk] (half-tile step; window start: x pair | y << 8 | z << 20 in the region)
   float* xk;    // two widths: [chunk][4 NK] d g_D along x, two pairs per float4
   float* xd;    // two widths: [chunk][2 NP] g_D along x
 };
@@ -320,8 +331,8 @@ __device__ inline PencilTables pencil_tables(float4* sm, int t) {
   s.zt = s.yt + C * MGT;
   s.pf = s.zt + C * MGT;
   s.pt = s.pf + C;
-  s.po = reinterpret_cast<int4*>(s.pt + C);
-  s.xk = reinterpret_cast<float*>(s.po + C);
+  s.po = reinterpret_cast<int2*>(s.pt + C);
+  s.xk = reinterpret_cast<float*>(s.pt + 2 * C);
   s.xd = s.xk + C * 4 * NK;
   return s;
 }
@@ -355,53 +366,101 @@ __device__ __forceinline__ void pencil_fetch(float4* r, int base, int np, const 
 
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
-template <int OXP, int NP, int EXT2, int MODE>
-__device__ __forceinline__ void pencil_row(const float4* __restrict__ xa, const float4* __restrict__ xb,
-                                           const float4* __restrict__ xk, const float2* __restrict__ xd,
-                                           float2 (&sx)[EXT2], float2 (&sy)[EXT2], float2 (&sz)[EXT2],
-                                           float c0, float c1, float c2, float c3, float c4, float c5,
-                                           float c6, float c7, float c8, float c9, float c10) {
+// Register sums of one grid row (three components, EXT2 point pairs).
+template <int EXT2>
+struct PencilRow {
+  float2 x[EXT2], y[EXT2], z[EXT2];
+};
+
+// Coefficients of one row and particle (all zero, or P and B with G F' = 0, outside the window):
+// same width G, G alpha (3); forces P, B, G F' (3); two widths a, b, c (3 each), k_y, k_z.
+template <int MODE>
+struct PencilCoef {
+  static constexpr int N = MODE == kPencilSameWidth ? 4 : (MODE == kPencilForces ? 5 : 11);
+  float2 c[N];   // each value twice, the packed instructions' operands
+};
+
+template <int MODE>
+__device__ __forceinline__ PencilCoef<MODE> pencil_coef(const KernelConsts<float>& kc, float4 yv, float4 zv, float4 f,
+                                                        float4 u, bool in) {
+  PencilCoef<MODE> r;
+  const float P = yv.z + zv.z;
+  const float dy = yv.y, dz = zv.y;
+  if constexpr (MODE == kPencilSameWidth) {
+    const float G = in ? yv.x * zv.x : 0.f;
+    r.c[0] = dup2(G);
+    r.c[1] = dup2(G * fmaf(f.x, P, fmaf(u.y, dz, -u.z * dy)));
+    r.c[2] = dup2(G * fmaf(f.y, P, -u.x * dz));
+    r.c[3] = dup2(G * fmaf(f.z, P, u.x * dy));
+  } else if constexpr (MODE == kPencilForces) {
+    const float G = in ? yv.x * zv.x : 0.f;
+    r.c[0] = dup2(P);
+    r.c[1] = dup2(kc.B);
+    r.c[2] = dup2(G * f.x);
+    r.c[3] = dup2(G * f.y);
+    r.c[4] = dup2(G * f.z);
+  } else {
+    const float G = in ? kc.nrm * yv.x * zv.x : 0.f;
+    const float GQ = G * P, GB = G * kc.B;
+    const float H = in ? kc.tq * yv.w * zv.w : 0.f;
+    r.c[0] = dup2(f.x * GQ); r.c[1] = dup2(f.y * GQ); r.c[2] = dup2(f.z * GQ);
+    r.c[3] = dup2(f.x * GB); r.c[4] = dup2(f.y * GB); r.c[5] = dup2(f.z * GB);
+    r.c[6] = dup2(H * (u.y * dz - u.z * dy));
+    r.c[7] = dup2(-H * u.x * dz);
+    r.c[8] = dup2(H * u.x * dy);
+    r.c[9] = dup2(H * u.z);
+    r.c[10] = dup2(-H * u.y);
+  }
+  return r;
+}
+
+// One point pair of one row.
+template <int MODE, int K, int EXT2>
+__device__ __forceinline__ void pencil_pair(PencilRow<EXT2>& s, const PencilCoef<MODE>& r, float4 p0, float4 p1,
+                                            float2 k2, float2 d2) {
+  const float2* c = r.c;
+  const float2 g2 = make_float2(p0.x, p0.y), q2 = make_float2(p0.z, p0.w);
+  if constexpr (MODE == kPencilSameWidth) {
+    s.x[K] = __ffma2_rn(c[0], q2, __ffma2_rn(c[1], g2, s.x[K]));
+    s.y[K] = __ffma2_rn(c[0], make_float2(p1.x, p1.y), __ffma2_rn(c[2], g2, s.y[K]));
+    s.z[K] = __ffma2_rn(c[0], make_float2(p1.z, p1.w), __ffma2_rn(c[3], g2, s.z[K]));
+  } else if constexpr (MODE == kPencilForces) {
+    const float2 w = __ffma2_rn(c[1], q2, __fmul2_rn(c[0], g2));
+    s.x[K] = __ffma2_rn(c[2], w, s.x[K]);
+    s.y[K] = __ffma2_rn(c[3], w, s.y[K]);
+    s.z[K] = __ffma2_rn(c[4], w, s.z[K]);
+  } else {
+    const float2 vx = __ffma2_rn(c[3], q2, __ffma2_rn(c[0], g2, s.x[K]));
+    float2 vy = __ffma2_rn(c[4], q2, __ffma2_rn(c[1], g2, s.y[K]));
+    float2 vz = __ffma2_rn(c[5], q2, __ffma2_rn(c[2], g2, s.z[K]));
+    vy = __ffma2_rn(c[9], k2, vy);
+    vz = __ffma2_rn(c[10], k2, vz);
+    s.x[K] = __ffma2_rn(c[6], d2, vx);
+    s.y[K] = __ffma2_rn(c[7], d2, vy);
+    s.z[K] = __ffma2_rn(c[8], d2, vz);
+  }
+}
+
+// A particle's update of the thread's R rows: each profile is read once for all.
+template <int R, int OXP, int JP, int NP, int EXT2, int MODE>
+__device__ __forceinline__ void pencil_rows(const float4* __restrict__ xa, const float4* __restrict__ xb,
+                                            const float4* __restrict__ xk, const float2* __restrict__ xd, float4 k4,
+                                            PencilRow<EXT2>& s0, PencilRow<EXT2>& s1, const PencilCoef<MODE>& r0,
+                                            const PencilCoef<MODE>& r1) {
   static_assert(OXP + NP <= EXT2, "pair window beyond the row");
-  if (MODE == kPencilSameWidth) {   // c0 = G, c1..c3 = G alpha
-    const float2 G2 = dup2(c0), AX = dup2(c1), AY = dup2(c2), AZ = dup2(c3);
-#pragma unroll
-    for (int jp = 0; jp < NP; ++jp) {
-      const float4 p0 = xa[jp], p1 = xb[jp];
-      const float2 g2 = make_float2(p0.x, p0.y);
-      sx[OXP + jp] = __ffma2_rn(G2, make_float2(p0.z, p0.w), __ffma2_rn(AX, g2, sx[OXP + jp]));
-      sy[OXP + jp] = __ffma2_rn(G2, make_float2(p1.x, p1.y), __ffma2_rn(AY, g2, sy[OXP + jp]));
-      sz[OXP + jp] = __ffma2_rn(G2, make_float2(p1.z, p1.w), __ffma2_rn(AZ, g2, sz[OXP + jp]));
+  if constexpr (JP < NP) {
+    const float4 p0 = xa[JP];
+    float4 p1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 k2 = make_float2(0.f, 0.f), d2 = make_float2(0.f, 0.f);
+    if constexpr (MODE == kPencilSameWidth) p1 = xb[JP];
+    if constexpr (MODE == kPencilTwoWidths) {
+      if constexpr ((JP & 1) == 0) k4 = xk[JP >> 1];
+      k2 = (JP & 1) ? make_float2(k4.z, k4.w) : make_float2(k4.x, k4.y);
+      d2 = xd[JP];
     }
-  } else if (MODE == kPencilForces) {   // c0 = P, c1 = B, c2..c4 = G F'
-    const float2 P2 = dup2(c0), B2 = dup2(c1), FX = dup2(c2), FY = dup2(c3), FZ = dup2(c4);
-#pragma unroll
-    for (int jp = 0; jp < NP; ++jp) {
-      const float4 p0 = xa[jp];
-      const float2 w = __ffma2_rn(B2, make_float2(p0.z, p0.w), __fmul2_rn(P2, make_float2(p0.x, p0.y)));
-      sx[OXP + jp] = __ffma2_rn(FX, w, sx[OXP + jp]);
-      sy[OXP + jp] = __ffma2_rn(FY, w, sy[OXP + jp]);
-      sz[OXP + jp] = __ffma2_rn(FZ, w, sz[OXP + jp]);
-    }
-  } else {   // two widths: c0..c2 = a, c3..c5 = b, c6..c8 = c, c9 = ky, c10 = kz
-    const float2 AX = dup2(c0), AY = dup2(c1), AZ = dup2(c2), BX = dup2(c3), BY = dup2(c4), BZ = dup2(c5);
-    const float2 CX = dup2(c6), CY = dup2(c7), CZ = dup2(c8), KY = dup2(c9), KZ = dup2(c10);
-    float4 k4 = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int jp = 0; jp < NP; ++jp) {
-      const float4 p0 = xa[jp];
-      const float2 g2 = make_float2(p0.x, p0.y), q2 = make_float2(p0.z, p0.w);
-      if ((jp & 1) == 0) k4 = xk[jp >> 1];
-      const float2 k2 = (jp & 1) ? make_float2(k4.z, k4.w) : make_float2(k4.x, k4.y);
-      const float2 d2 = xd[jp];
-      float2 vx = __ffma2_rn(BX, q2, __ffma2_rn(AX, g2, sx[OXP + jp]));
-      float2 vy = __ffma2_rn(BY, q2, __ffma2_rn(AY, g2, sy[OXP + jp]));
-      float2 vz = __ffma2_rn(BZ, q2, __ffma2_rn(AZ, g2, sz[OXP + jp]));
-      vy = __ffma2_rn(KY, k2, vy);
-      vz = __ffma2_rn(KZ, k2, vz);
-      sx[OXP + jp] = __ffma2_rn(CX, d2, vx);
-      sy[OXP + jp] = __ffma2_rn(CY, d2, vy);
-      sz[OXP + jp] = __ffma2_rn(CZ, d2, vz);
-    }
+    pencil_pair<MODE, OXP + JP>(s0, r0, p0, p1, k2, d2);
+    if constexpr (R == 2) pencil_pair<MODE, OXP + JP>(s1, r1, p0, p1, k2, d2);
+    pencil_rows<R, OXP, JP + 1, NP, EXT2, MODE>(xa, xb, xk, xd, k4, s0, s1, r0, r1);
   }
 }
 
@@ -430,14 +489,27 @@ __device__ __forceinline__ void pencil_flush(int x0, int Mx, bool vec_rows, floa
   }
 }
 
+// The same pairs of a row's three components (Mtot reals apart).
 template <int EXT2>
-__device__ __forceinline__ void pencil_shift(float2 (&s)[EXT2]) {
-#pragma unroll
-  for (int k = 0; k < EXT2; ++k) s[k] = (k + 2 < EXT2) ? s[k + 2] : make_float2(0.f, 0.f);
+__device__ __forceinline__ void pencil_flush3(int x0, int Mx, bool vec_rows, float* __restrict__ row, size_t Mtot,
+                                              const PencilRow<EXT2>& s, int k0, int k1) {
+  pencil_flush<EXT2>(x0, Mx, vec_rows, row, s.x, k0, k1);
+  pencil_flush<EXT2>(x0, Mx, vec_rows, row + Mtot, s.y, k0, k1);
+  pencil_flush<EXT2>(x0, Mx, vec_rows, row + 2 * Mtot, s.z, k0, k1);
 }
 
-template <int MGT, bool GUARD, int MODE>
-__global__ void __launch_bounds__(rows_threads(MGT), 1) spread_pencil_kernel(Geometry<float> g, KernelConsts<float> kc,
+template <int EXT2>
+__device__ __forceinline__ void pencil_shift(PencilRow<EXT2>& s) {
+#pragma unroll
+  for (int k = 0; k < EXT2; ++k) {
+    s.x[k] = (k + 2 < EXT2) ? s.x[k + 2] : make_float2(0.f, 0.f);
+    s.y[k] = (k + 2 < EXT2) ? s.y[k + 2] : make_float2(0.f, 0.f);
+    s.z[k] = (k + 2 < EXT2) ? s.z[k + 2] : make_float2(0.f, 0.f);
+  }
+}
+
+template <int MGT, bool GUARD, int MODE, int R>
+__global__ void __launch_bounds__(pencil_threads(MGT, R), R) spread_pencil_kernel(Geometry<float> g, KernelConsts<float> kc,
                                                                           const float4* __restrict__ pos,
                                                                           const float4* __restrict__ Fv,
                                                                           const float4* __restrict__ Tv,
@@ -462,17 +534,30 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_pencil_kernel(Geo
   const int oy0 = (pc % nty) * g.tile[1], oz0 = (pc / nty) * g.tile[2];
   const int MG = GUARD ? g.MG : MGT;
   const int EY = g.tile[1] + MG - 1, EZ = g.tile[2] + MG - 1;
-  const int row = threadIdx.x;
-  const bool has_row = row < EY * EZ;
-  const int ez = has_row ? row / EY : 0;
-  const int ey = has_row ? row - ez * EY : 0;
-  float2 sx[EXT2], sy[EXT2], sz[EXT2];
+  // the thread's rows R t .. R t + R - 1 (numbered ey + EY ez)
+  const int row = R * threadIdx.x;
+  const bool has0 = row < EY * EZ, has1 = R == 2 && row + 1 < EY * EZ;
+  const int ez0 = has0 ? row / EY : 0, ey0 = has0 ? row - ez0 * EY : 0;
+  const int ez1 = has1 ? (row + 1) / EY : 0, ey1 = has1 ? row + 1 - ez1 * EY : 0;
+  PencilRow<EXT2> s0r, s1r;
 #pragma unroll
   for (int k = 0; k < EXT2; ++k) {
-    sx[k] = make_float2(0.f, 0.f);
-    sy[k] = make_float2(0.f, 0.f);
-    sz[k] = make_float2(0.f, 0.f);
+    s0r.x[k] = s0r.y[k] = s0r.z[k] = make_float2(0.f, 0.f);
+    s1r.x[k] = s1r.y[k] = s1r.z[k] = make_float2(0.f, 0.f);
   }
+  const bool vec_rows = (g.M[0] & 3) == 0;
+  // adds pairs [0, k1) of both rows to the grid, x from 4 c on
+  auto flush = [&](int c, int k1) {
+    const size_t Mtot = (size_t)g.M[0] * g.M[1] * g.M[2];
+    if (has0) {
+      float* r = grid + ((size_t)wrap_index(oz0 + ez0, g.M[2]) * g.M[1] + wrap_index(oy0 + ey0, g.M[1])) * g.M[0];
+      pencil_flush3<EXT2>(4 * c, g.M[0], vec_rows, r, Mtot, s0r, 0, k1);
+    }
+    if (has1) {
+      float* r = grid + ((size_t)wrap_index(oz0 + ez1, g.M[2]) * g.M[1] + wrap_index(oy0 + ey1, g.M[1])) * g.M[0];
+      pencil_flush3<EXT2>(4 * c, g.M[0], vec_rows, r, Mtot, s1r, 0, k1);
+    }
+  };
   int cur = 2 * s0;   // half-tile step whose x origin (4 cur) anchors the register row
   constexpr int C = pencil_chunk(MGT, MODE);
   // profile tables of one pass (particles [base, base + np)) from its raw rows
@@ -535,12 +620,9 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_pencil_kernel(Geo
       const int wx = wrap_once(i0.x, g.M[0]);
       const int step = min(max(wx >> 3, 0), ntx - 1);
       const int ox = min(max(wx - 8 * step, 0), 7);   // the binning's half of the tile: ox >= 4
-      int4 off;
-      off.x = ox & 3;
-      off.y = min(max(wrap_once(i0.y, g.M[1]) - oy0, 0), g.tile[1] - 1);
-      off.z = min(max(wrap_once(i0.z, g.M[2]) - oz0, 0), g.tile[2] - 1);
-      off.w = 2 * step + (ox >> 2);
-      tb.po[q] = off;
+      const int wy = min(max(wrap_once(i0.y, g.M[1]) - oy0, 0), g.tile[1] - 1);
+      const int wz = min(max(wrap_once(i0.z, g.M[2]) - oz0, 0), g.tile[2] - 1);
+      tb.po[q] = make_int2(2 * step + (ox >> 2), ((ox & 3) >> 1) | (wy << 8) | (wz << 20));
       const float4 f = rF[q];
       const float4 t = TORQUE ? rT[q] : make_float4(0.f, 0.f, 0.f, 0.f);
       if (MODE == kPencilTwoWidths) {
@@ -566,76 +648,70 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_pencil_kernel(Geo
     if (pass + 2 < npass)
       pencil_fetch<TORQUE, C>(pencil_raw<MGT, MODE>(sm4, pass & 1), base + 2 * C, min(C, p_end - base - 2 * C), pos, Fv, Tv);
     const PencilTables tb = pencil_tables<MGT, MODE>(sm4, pass & 1);
-    for (int q = 0; q < np; ++q) {
-      const int4 off = tb.po[q];
-      // the walk reaches the particle's half tile: complete points of the passed half tiles go to the grid
-      while (cur < off.w) {
-        if (has_row) {
-          const size_t Mtot = (size_t)g.M[0] * g.M[1] * g.M[2];
-          float* r0 = grid + ((size_t)wrap_index(oz0 + ez, g.M[2]) * g.M[1] + wrap_index(oy0 + ey, g.M[1])) * g.M[0];
-          const bool vec_rows = (g.M[0] & 3) == 0;
-          pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0, sx, 0, 2);
-          pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0 + Mtot, sy, 0, 2);
-          pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0 + 2 * Mtot, sz, 0, 2);
-        }
-        pencil_shift<EXT2>(sx);
-        pencil_shift<EXT2>(sy);
-        pencil_shift<EXT2>(sz);
-        ++cur;
-      }
-      const int jy = ey - off.y, jz = ez - off.z;
-      const bool in = has_row && (unsigned)jy < (unsigned)MG && (unsigned)jz < (unsigned)MG;
-      if (!__any_sync(kFullMask32, in)) continue;
-      const float4 yv = tb.yt[q * MGT + (in ? jy : 0)];
-      const float4 zv = tb.zt[q * MGT + (in ? jz : 0)];
+    int2 off;
+    bool act;
+    PencilCoef<MODE> r0, r1;
+    // particle q's place and row coefficients; whether any row of the warp is in its window
+    auto prep = [&](int q, int2& o, PencilCoef<MODE>& a, PencilCoef<MODE>& b) -> bool {
+      if (R == 2) o = tb.po[q];
+      const int wy = (o.y >> 8) & 0xfff, wz = o.y >> 20;
+      const int jy0 = ey0 - wy, jz0 = ez0 - wz, jy1 = ey1 - wy, jz1 = ez1 - wz;
+      const bool in0 = has0 && (unsigned)jy0 < (unsigned)MG && (unsigned)jz0 < (unsigned)MG;
+      const bool in1 = has1 && (unsigned)jy1 < (unsigned)MG && (unsigned)jz1 < (unsigned)MG;
+      if (R == 1 && !__any_sync(kFullMask32, in0)) return false;
+      const float4* yt = tb.yt + q * MGT;
+      const float4* zt = tb.zt + q * MGT;
       const float4 f = tb.pf[q];
-      const float P = yv.z + zv.z;
-      float c[11];
-      if (MODE == kPencilSameWidth) {
-        const float4 u = tb.pt[q];
-        const float G = in ? yv.x * zv.x : 0.f;
-        const float dy = yv.y, dz = zv.y;
-        c[0] = G;
-        c[1] = G * fmaf(f.x, P, fmaf(u.y, dz, -u.z * dy));
-        c[2] = G * fmaf(f.y, P, -u.x * dz);
-        c[3] = G * fmaf(f.z, P, u.x * dy);
-        for (int k = 4; k < 11; ++k) c[k] = 0.f;
-      } else if (MODE == kPencilForces) {
-        const float G = in ? yv.x * zv.x : 0.f;
-        c[0] = P;
-        c[1] = kc.B;
-        c[2] = G * f.x;
-        c[3] = G * f.y;
-        c[4] = G * f.z;
-        for (int k = 5; k < 11; ++k) c[k] = 0.f;
-      } else {
-        const float4 tq = tb.pt[q];
-        const float G = in ? kc.nrm * yv.x * zv.x : 0.f;
-        const float GQ = G * P, GB = G * kc.B;
-        const float H = in ? kc.tq * yv.w * zv.w : 0.f;
-        const float dy = yv.y, dz = zv.y;
-        c[0] = f.x * GQ; c[1] = f.y * GQ; c[2] = f.z * GQ;
-        c[3] = f.x * GB; c[4] = f.y * GB; c[5] = f.z * GB;
-        c[6] = H * (tq.y * dz - tq.z * dy);
-        c[7] = -H * tq.x * dz;
-        c[8] = H * tq.x * dy;
-        c[9] = H * tq.z;
-        c[10] = -H * tq.y;
+      const float4 u = TORQUE ? tb.pt[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+      a = pencil_coef<MODE>(kc, yt[in0 ? jy0 : 0], zt[in0 ? jz0 : 0], f, u, in0);
+      if constexpr (R == 2) {
+        b = pencil_coef<MODE>(kc, yt[in1 ? jy1 : 0], zt[in1 ? jz1 : 0], f, u, in1);
+        return __any_sync(kFullMask32, in0 || in1);
+      }
+      return true;
+    };
+    // Two rows: a software pipeline. While the FMAs of particle q run, the loads and the row coefficients of
+    // q + 1 are under way in the same instruction stream.
+    if (R == 2) {
+      act = prep(0, off, r0, r1);
+    }
+    for (int q = 0; q < np; ++q) {
+      if (R == 1) off = tb.po[q];
+      // the walk reaches the particle's half tile: complete points of the passed half tiles go to the grid
+      while (cur < off.x) {
+        flush(cur, 2);
+        pencil_shift<EXT2>(s0r);
+        if (R == 2) pencil_shift<EXT2>(s1r);
+        ++cur;
       }
       const float4* xa = tb.xa + (size_t)q * NP;
       const float4* xb = tb.xb + (size_t)q * NP;
       const float4* xk = reinterpret_cast<const float4*>(tb.xk + (size_t)q * 4 * NK);
       const float2* xd = reinterpret_cast<const float2*>(tb.xd + (size_t)q * 2 * NP);
-#define FCM_PENCIL_CASE(OXP)                                                                                    \
-  case OXP:                                                                                                     \
-    pencil_row<OXP, NP, EXT2, MODE>(xa, xb, xk, xd, sx, sy, sz, c[0], c[1], c[2], c[3], c[4], c[5], c[6], c[7], \
-                                    c[8], c[9], c[10]);                                                         \
-    break;
-      switch (off.x >> 1) {
-        FCM_PENCIL_CASE(0) FCM_PENCIL_CASE(1)
-        default: break;
+      const float4 k4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (R == 1) {
+        if (!prep(q, off, r0, r1)) continue;
+        if (off.y & 1) pencil_rows<R, 1, 0, NP, EXT2, MODE>(xa, xb, xk, xd, k4, s0r, s1r, r0, r1);
+        else pencil_rows<R, 0, 0, NP, EXT2, MODE>(xa, xb, xk, xd, k4, s0r, s1r, r0, r1);
+      } else {
+        const int qn = min(q + 1, np - 1);
+        int2 offn;
+        PencilCoef<MODE> n0, n1;
+        bool actn;
+        if (!act) {
+          actn = prep(qn, offn, n0, n1);
+        } else if (off.y & 1) {
+          actn = prep(qn, offn, n0, n1);
+          pencil_rows<R, 1, 0, NP, EXT2, MODE>(xa, xb, xk, xd, k4, s0r, s1r, r0, r1);
+        } else {
+          actn = prep(qn, offn, n0, n1);
+          pencil_rows<R, 0, 0, NP, EXT2, MODE>(xa, xb, xk, xd, k4, s0r, s1r, r0, r1);
+        }
+        off = offn;
+        act = actn;
+        r0 = n0;
+        r1 = n1;
       }
-#undef FCM_PENCIL_CASE
     }
     // tables of the next pass, into the set the previous pass used
     if (pass + 1 < npass)
@@ -643,14 +719,7 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_pencil_kernel(Geo
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();   // the next tables and the raw rows of pass + 2 are in; this pass's tables are free
   }
-  if (has_row) {   // the last tile reached: every pair of the register row, x from 8 cur on
-    const size_t Mtot = (size_t)g.M[0] * g.M[1] * g.M[2];
-    float* r0 = grid + ((size_t)wrap_index(oz0 + ez, g.M[2]) * g.M[1] + wrap_index(oy0 + ey, g.M[1])) * g.M[0];
-    const bool vec_rows = (g.M[0] & 3) == 0;
-    pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0, sx, 0, EXT2);
-    pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0 + Mtot, sy, 0, EXT2);
-    pencil_flush<EXT2>(4 * cur, g.M[0], vec_rows, r0 + 2 * Mtot, sz, 0, EXT2);
-  }
+  flush(cur, EXT2);   // the last half tile reached: every pair of the register rows
 }
 
 // ---------------------------------------------------------------- atomic kernel
@@ -784,11 +853,21 @@ static bool rows_selected(const Geometry<float>& g, int spread_kernel) {
   return spread_uses_rows(g.tile, g.MG);
 }
 
+template <int MGT, bool GUARD, int MODE, int R>
+static void pencil_launch(const Geometry<float>& g, const KernelConsts<float>& kc, const BinBuffers& b, float* grid,
+                          cudaStream_t s, int blocks, int segl) {
+  const size_t smem = pencil_tables_bytes(MGT, MODE);
+  const int rows = (g.tile[1] + g.MG - 1) * (g.tile[2] + g.MG - 1);
+  const int threads = (((rows + R - 1) / R + 31) / 32) * 32;
+  auto k = spread_pencil_kernel<MGT, GUARD, MODE, R>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k<<<blocks, threads, smem, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F, (const float4*)b.t_T,
+                                  b.tile_start, grid, segl);
+}
+
 template <int MGT, bool GUARD, int MODE>
 static void pencil_variant(const Geometry<float>& g, const KernelConsts<float>& kc, const BinBuffers& b, float* grid,
                            cudaStream_t s) {
-  const size_t smem = pencil_tables_bytes(MGT, MODE);
-  const int threads = (((g.tile[1] + g.MG - 1) * (g.tile[2] + g.MG - 1) + 31) / 32) * 32;
   const int nsys = g.nsys > 1 ? g.nsys : 1;
   const int pencils = nsys * g.ntile[1] * g.ntile[2];
   // Long pencils are split into segments when there are too few pencils for four waves of one CTA per SM
@@ -796,10 +875,10 @@ static void pencil_variant(const Geometry<float>& g, const KernelConsts<float>& 
   const int nseg = std::min(g.ntile[0], std::max(1, (4 * device_sm_count() + pencils - 1) / pencils));
   const int segl = (g.ntile[0] + nseg - 1) / nseg;
   const int blocks = pencils * ((g.ntile[0] + segl - 1) / segl);
-  auto k = spread_pencil_kernel<MGT, GUARD, MODE>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k<<<blocks, threads, smem, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F, (const float4*)b.t_T,
-                                  b.tile_start, grid, segl);
+  if constexpr (pencil_two_rows(MGT, MODE)) {
+    if (blocks > device_sm_count()) return pencil_launch<MGT, GUARD, MODE, 2>(g, kc, b, grid, s, blocks, segl);
+  }
+  pencil_launch<MGT, GUARD, MODE, 1>(g, kc, b, grid, s, blocks, segl);
 }
 
 size_t spread_smem_bytes(const int tile[3], int MG) {
