@@ -17,8 +17,179 @@
 
 namespace fcm {
 
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+
+// One halving step of a warp sum over two values: lanes with bit `s` clear keep the sum of a, the
+// others that of b (one shuffle for both; each value's additions are those of the butterfly).
+__device__ __forceinline__ float fold2(float a, float b, int s, bool hi) {
+  return (hi ? b : a) + __shfl_xor_sync(kFullMask32, hi ? a : b, s);
+}
+
+__device__ __forceinline__ float fold1(float a, int s) { return a + __shfl_xor_sync(kFullMask32, a, s); }
+
+// Sums over the warp's lanes, times h^3, to row `i` of U and W (plus the pair sums, where given). The sum
+// halves its values as it goes: 8 shuffles for six values, 6 for three, instead of 30 and 15.
+template <bool TORQUE>
+__device__ __forceinline__ void gather_store(int lane, int i, float h3, float u0, float u1, float u2, float w0,
+                                             float w1, float w2, const float* __restrict__ upair,
+                                             const float* __restrict__ wpair, float* __restrict__ U,
+                                             float* __restrict__ W) {
+  const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+  const size_t oi = 3 * (size_t)i;
+  if (TORQUE) {
+    const float v0 = fold2(u0, w0, 16, b16), v1 = fold2(u1, w1, 16, b16), v2 = fold2(u2, w2, 16, b16);
+    const float v = fold1(fold1(fold2(fold2(v0, v1, 8, b8), fold1(v2, 8), 4, b4), 2), 1);
+    const int c = b4 ? 2 : (b8 ? 1 : 0);   // lanes 0, 8, 4 hold U, lanes 16, 24, 20 W
+    float* out = b16 ? W : U;
+    const float* add = b16 ? wpair : upair;
+    if ((lane & 3) == 0 && !(b4 && b8) && out) out[oi + c] = h3 * v + (add ? add[oi + c] : 0.f);
+  } else {
+    const float v = fold1(fold1(fold1(fold2(fold2(u0, u1, 16, b16), fold1(u2, 16), 8, b8), 4), 2), 1);
+    const int c = b8 ? 2 : (b16 ? 1 : 0);   // lanes 0, 16, 8
+    if ((lane & 7) == 0 && !(b8 && b16)) U[oi + c] = h3 * v + (upair ? upair[oi + c] : 0.f);
+  }
+}
+
+// One particle's sums (each lane's part) with torques, one width and a compiled support, in packed FMAs: with
+// S = sum_x g u along a row and T(x) = sum_rows G u down a column (G = g(dy) g(dz)), six FMAs per window point,
+//   U = nrm (sum_rows G P S + B sum_x d^2 g T),  P = A + B (dy^2 + dz^2),
+//   W = tq  (sum_rows G (dy S_z - dz S_y, dz S_x, -dy S_x) + sum_x d g (0, -T_z, T_y)).
+// The general form's eight FMAs per point were 43% of the kernel's instructions, at 65% of the issue slots
+// (M_G = 14): 363 M -> 268 M warp instructions for 3 x 65,536 particles.
+template <int MGT>
+__device__ __forceinline__ void gather_particle(const Geometry<float>& g, const KernelConsts<float>& kc,
+                                                const ExtLayout& l, const float* acc, int zs,
+                                                const TileOrigin& o, int lane, float4 y, float& u0, float& u1,
+                                                float& u2, float& w0, float& w1, float& w2) {
+  const int ring = l.EZ;
+  const int3 i0 = window_starts(g, y);
+  const int4 off = window_offset(g, o, i0);
+  const float dxl = (float)(i0.x + lane) * g.h[0] - y.x;
+  const float dyl = (float)(i0.y + lane) * g.h[1] - y.y;
+  const float dzl = (float)(i0.z + lane) * g.h[2] - y.z;
+  const float gxl = expf(-dxl * dxl * kc.inv2S2);
+  const float gyl = expf(-dyl * dyl * kc.inv2S2);
+  const float gzl = expf(-dzl * dzl * kc.inv2S2);
+  u0 = u1 = u2 = w0 = w1 = w2 = 0.f;
+  float2 gg[MGT], gp[MGT / 2];       // g(x) twice; of two points
+  float2 tyz[MGT], tx[MGT / 2];      // column sums of (u_y, u_z); of u_x at two points
+#pragma unroll
+  for (int j = 0; j < MGT; ++j) {
+    gg[j] = dup2(__shfl_sync(kFullMask32, gxl, j));
+    tyz[j] = make_float2(0.f, 0.f);
+  }
+#pragma unroll
+  for (int j = 0; j < MGT / 2; ++j) {
+    gp[j] = make_float2(gg[2 * j].x, gg[2 * j + 1].x);
+    tx[j] = make_float2(0.f, 0.f);
+  }
+  int zb = zs + off.z;   // ring slot of the window's first plane
+  if (zb >= ring) zb -= ring;
+  const float* pbase = acc + off.y * l.P + off.x;
+  const float2* yzbase = reinterpret_cast<const float2*>(acc + yz_plane_offset(l)) + off.y * l.P + off.x;
+  constexpr int NFULL = MGT * MGT / 32, TAIL = MGT * MGT % 32;
+  constexpr bool SPLIT_TAIL = TAIL > 0 && TAIL * MGT <= 64;   // a short last pass: split it by points
+#pragma unroll
+  for (int it = 0; it < (SPLIT_TAIL ? NFULL : (MGT * MGT + 31) / 32); ++it) {
+    // window row r = jy + M_G jz of lane and pass it: fixed per lane
+    const int r = 32 * it + lane;
+    const bool active = r < MGT * MGT;
+    const int jz = active ? r / MGT : 0, jy = active ? r - (r / MGT) * MGT : 0;
+    int sl = zb + jz;
+    if (sl >= ring) sl -= ring;
+    const int ro = sl * l.Q + jy * l.P;
+    const float dy = __shfl_sync(kFullMask32, dyl, jy);
+    const float gy = __shfl_sync(kFullMask32, gyl, jy);
+    const float dz = __shfl_sync(kFullMask32, dzl, jz);
+    const float gz = __shfl_sync(kFullMask32, gzl, jz);
+    const float G = active ? gy * gz : 0.f;
+    const float2 G2 = dup2(G);
+    float2 sx = make_float2(0.f, 0.f), syz = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < MGT; j += 2) {
+      const float2 ux = make_float2(pbase[ro + j], pbase[ro + j + 1]);
+      const float2 ua = yzbase[ro + j], ub = yzbase[ro + j + 1];
+      sx = __ffma2_rn(gp[j / 2], ux, sx);
+      tx[j / 2] = __ffma2_rn(G2, ux, tx[j / 2]);
+      syz = __ffma2_rn(gg[j], ua, syz);
+      tyz[j] = __ffma2_rn(G2, ua, tyz[j]);
+      syz = __ffma2_rn(gg[j + 1], ub, syz);
+      tyz[j + 1] = __ffma2_rn(G2, ub, tyz[j + 1]);
+    }
+    const float s0 = sx.x + sx.y;
+    const float GP = G * fmaf(kc.B, fmaf(dy, dy, dz * dz), kc.A);
+    u0 = fmaf(GP, s0, u0);
+    u1 = fmaf(GP, syz.x, u1);
+    u2 = fmaf(GP, syz.y, u2);
+    const float Gs0 = G * s0;
+    w0 = fmaf(G, dy * syz.y - dz * syz.x, w0);
+    w1 = fmaf(dz, Gs0, w1);
+    w2 = fmaf(-dy, Gs0, w2);
+  }
+  if (SPLIT_TAIL) {
+    // the last TAIL rows have TAIL * M_G (row, point) items: each lane takes up to two and applies
+    // the row's y, z factors to each item itself
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {
+      const int e = lane + 32 * pass;
+      const bool valid = e < TAIL * MGT;
+      const int t = valid ? e / MGT : 0, j = valid ? e - (e / MGT) * MGT : 0;
+      const int r = 32 * NFULL + t;
+      const int jz = r / MGT, jy = r - jz * MGT;
+      const float gj = __shfl_sync(kFullMask32, gxl, j);
+      const float dj = __shfl_sync(kFullMask32, dxl, j);
+      const float dy = __shfl_sync(kFullMask32, dyl, jy);
+      const float gy = __shfl_sync(kFullMask32, gyl, jy);
+      const float dz = __shfl_sync(kFullMask32, dzl, jz);
+      const float gz = __shfl_sync(kFullMask32, gzl, jz);
+      if (valid) {
+        int sl = zb + jz;
+        if (sl >= ring) sl -= ring;
+        const int ro = sl * l.Q + jy * l.P + j;
+        const float ux = pbase[ro];
+        const float2 uyz = yzbase[ro];
+        const float g3 = gy * gz * gj;
+        const float wgt = g3 * fmaf(kc.B, fmaf(dj, dj, fmaf(dy, dy, dz * dz)), kc.A);
+        u0 = fmaf(wgt, ux, u0);
+        u1 = fmaf(wgt, uyz.x, u1);
+        u2 = fmaf(wgt, uyz.y, u2);
+        w0 = fmaf(g3, dy * uyz.y - dz * uyz.x, w0);
+        w1 = fmaf(g3, dz * ux - dj * uyz.y, w1);
+        w2 = fmaf(g3, dj * uyz.x - dy * ux, w2);
+      }
+    }
+  }
+  // the terms in d and d^2 along x, from the column sums
+  float2 qx = make_float2(0.f, 0.f), qyz = qx, kyz = qx;
+#pragma unroll
+  for (int j = 0; j < MGT; j += 2) {
+    const float2 da = dup2(__shfl_sync(kFullMask32, dxl, j)), db = dup2(__shfl_sync(kFullMask32, dxl, j + 1));
+    const float2 ka = __fmul2_rn(da, gg[j]), kb = __fmul2_rn(db, gg[j + 1]);
+    const float2 qa = __fmul2_rn(da, ka), qb = __fmul2_rn(db, kb);
+    qx = __ffma2_rn(make_float2(qa.x, qb.x), tx[j / 2], qx);
+    qyz = __ffma2_rn(qa, tyz[j], qyz);
+    qyz = __ffma2_rn(qb, tyz[j + 1], qyz);
+    kyz = __ffma2_rn(ka, tyz[j], kyz);
+    kyz = __ffma2_rn(kb, tyz[j + 1], kyz);
+  }
+  u0 = kc.nrm * fmaf(kc.B, qx.x + qx.y, u0);
+  u1 = kc.nrm * fmaf(kc.B, qyz.x, u1);
+  u2 = kc.nrm * fmaf(kc.B, qyz.y, u2);
+  w0 *= kc.tq;
+  w1 = kc.tq * (w1 - kyz.y);
+  w2 = kc.tq * (w2 + kyz.x);
+}
+
+// CTAs per SM asked of the compiler: what the region's shared memory allows. Forces only with M_G = 10, three
+// (122,231 spheres on 216^3: 271 us, with two 312 us), with smaller supports more; from M_G = 12 on, and with
+// torques, two of 128 registers a thread (one of more registers: 32 x 65,536 spheres, M_G = 14, 5.76 against
+// 4.36 ms); the two largest supports' regions leave one.
+constexpr int gather_ctas(int MGT, bool guard, bool torque) {
+  return MGT > 16 ? 1 : (torque || (!guard && MGT >= 12) ? 2 : (MGT <= 8 ? 4 : 3));
+}
+
 template <int MGT, bool GUARD, bool TORQUE, bool SAMEW>
-__global__ void __launch_bounds__(256) gather_tile_kernel(Geometry<float> g, KernelConsts<float> kc,
+__global__ void __launch_bounds__(256, gather_ctas(MGT, GUARD, TORQUE)) gather_tile_kernel(Geometry<float> g, KernelConsts<float> kc,
                                                           const float4* __restrict__ pos,
                                                           const int* __restrict__ tstart,
                                                           const float* __restrict__ grid,
@@ -62,6 +233,12 @@ __global__ void __launch_bounds__(256) gather_tile_kernel(Geometry<float> g, Ker
 
     for (int p = p0 + warp; p < p1; p += nwarp) {
       const float4 y = pos[p];
+      float u0 = 0.f, u1 = 0.f, u2 = 0.f, w0 = 0.f, w1 = 0.f, w2 = 0.f;
+      if constexpr (!GUARD && TORQUE && SAMEW) {
+        gather_particle<MGT>(g, kc, l, acc, zs, o, lane, y, u0, u1, u2, w0, w1, w2);
+        gather_store<TORQUE>(lane, index_from_w(y.w), kc.h3, u0, u1, u2, w0, w1, w2, upair, wpair, U, W);
+        continue;
+      }
       const int3 i0 = window_starts(g, y);
       const int4 off = window_offset(g, o, i0);
       const float dxl = (float)(i0.x + lane) * g.h[0] - y.x;
@@ -84,7 +261,6 @@ __global__ void __launch_bounds__(256) gather_tile_kernel(Geometry<float> g, Ker
         gdx[j] = gdj;
         gx1[j] = dj * gdj;
       }
-      float u0 = 0.f, u1 = 0.f, u2 = 0.f, w0 = 0.f, w1 = 0.f, w2 = 0.f;
       // one window row (jy, jz) of this particle: x sums over the row, times the row's y, z factors
       auto row_update = [&](const float* row, int sy, int sz, bool active) {
         const float dy = __shfl_sync(kFullMask32, dyl, sy);
@@ -219,28 +395,7 @@ __global__ void __launch_bounds__(256) gather_tile_kernel(Geometry<float> g, Ker
           while (jy >= MG) { jy -= MG; ++jz; }
         }
       }
-#pragma unroll
-      for (int s = 16; s > 0; s >>= 1) {
-        u0 += __shfl_xor_sync(kFullMask32, u0, s);
-        u1 += __shfl_xor_sync(kFullMask32, u1, s);
-        u2 += __shfl_xor_sync(kFullMask32, u2, s);
-        if (TORQUE) {
-          w0 += __shfl_xor_sync(kFullMask32, w0, s);
-          w1 += __shfl_xor_sync(kFullMask32, w1, s);
-          w2 += __shfl_xor_sync(kFullMask32, w2, s);
-        }
-      }
-      if (lane == 0) {
-        const size_t oi = 3 * (size_t)index_from_w(y.w);
-        float a0 = kc.h3 * u0, a1 = kc.h3 * u1, a2 = kc.h3 * u2;
-        if (upair) { a0 += upair[oi]; a1 += upair[oi + 1]; a2 += upair[oi + 2]; }
-        U[oi] = a0; U[oi + 1] = a1; U[oi + 2] = a2;
-        if (TORQUE && W) {
-          float b0 = kc.h3 * w0, b1 = kc.h3 * w1, b2 = kc.h3 * w2;
-          if (wpair) { b0 += wpair[oi]; b1 += wpair[oi + 1]; b2 += wpair[oi + 2]; }
-          W[oi] = b0; W[oi + 1] = b1; W[oi + 2] = b2;
-        }
-      }
+      gather_store<TORQUE>(lane, index_from_w(y.w), kc.h3, u0, u1, u2, w0, w1, w2, upair, wpair, U, W);
     }
   }
 }

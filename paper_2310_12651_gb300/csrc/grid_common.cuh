@@ -91,48 +91,34 @@ __device__ inline int4 window_offset(const Geometry<float>& g, const TileOrigin&
 __host__ __device__ inline int yz_plane_offset(const ExtLayout& l) { return (l.C + 1) & ~1; }
 
 // Copies z planes [pa, pb) of the extended region of the grid (3 components) into shared memory
-// with asynchronous 4-byte copies: warps take (component, z) planes, lanes take x, rows advance by
-// pointer increments (the y range is split at its periodic wrap, so no per-row wrap test). Plane
-// ez is taken at grid z = o.oz0 + ez and goes to plane slot ez mod E_Z, so a CTA that walks a
-// z-pencil of tiles keeps the region as a ring of E_Z planes and copies only the planes a step
-// adds (pa, pb may exceed E_Z there; the default copies the whole region). Layout: the x component
-// as one plane (index slot Q + ey P + ex), then the y and z components interleaved as float2 at
-// the same index from yz_plane_offset, so the gather reads them with one 8-byte load.
+// with asynchronous 4-byte copies, waited for by each thread: threads take points of the (x, y) plane
+// and walk the planes and components, so a point's wraps and offsets are formed once for 3 (pb - pa)
+// copies and the lanes are full (a lane per x point left 11 of 32 idle at M_G = 14). Plane ez is taken
+// at grid z = o.oz0 + ez and goes to plane slot ez mod E_Z, so a CTA that walks a z-pencil of tiles
+// keeps the region as a ring of E_Z planes and copies only the planes a step adds (pa, pb may exceed
+// E_Z there). Layout: the x component as one plane (index slot Q + ey P + ex), then the y and z
+// components interleaved as float2 at the same index from yz_plane_offset, so the gather reads them
+// with one 8-byte load.
 __device__ inline void stage_region_async(const Geometry<float>& g, const TileOrigin& o, const ExtLayout& l,
-                                          const float* __restrict__ grid, float* ext, int pa = 0, int pb = -1) {
-  if (pb < 0) pb = l.EZ;
-  const size_t Mtot = (size_t)g.M[0] * g.M[1] * g.M[2];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  const int np = pb - pa;
-  if (lane < l.EX && np > 0) {
-    const int gx = wrap_index(o.ox0 + lane, g.M[0]);
-    const int gy0 = wrap_index(o.oy0, g.M[1]);
-    const int n1 = min(l.EY, g.M[1] - gy0);   // rows before the periodic wrap in y
-    const size_t row = (size_t)g.M[0];
-    for (int pl = warp; pl < 3 * np; pl += nwarp) {
-      const int c = pl >= 2 * np ? 2 : (pl >= np ? 1 : 0);
-      const int ez = pa + (pl - c * np);
-      const int gz = wrap_index(o.oz0 + ez, g.M[2]);
-      const int slot = ez % l.EZ;
-      const float* gplane = grid + c * Mtot + (size_t)gz * g.M[1] * g.M[0] + gx;
-      const int idx = slot * l.Q + lane;
-      float* dst = c == 0 ? ext + idx : ext + yz_plane_offset(l) + 2 * idx + (c - 1);
-      unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-      const unsigned sstep = (c == 0 ? 4u : 8u) * (unsigned)l.P;
-      // rows gy0 .. gy0 + n1 - 1, then rows 0 .. EY - n1 - 1: pointers advance by one row each
-      const float* src = gplane + (size_t)gy0 * row;
+                                          const float* __restrict__ grid, float* ext, int pa, int pb) {
+  const size_t plane = (size_t)g.M[0] * g.M[1], Mtot = plane * g.M[2];
+  const int s0 = pa % l.EZ, z0 = wrap_index(o.oz0 + pa, g.M[2]);
+  for (int e = threadIdx.x; e < l.EX * l.EY; e += blockDim.x) {
+    const int ey = e / l.EX, ex = e - ey * l.EX;
+    const float* src = grid + (size_t)wrap_index(o.oy0 + ey, g.M[1]) * g.M[0] + wrap_index(o.ox0 + ex, g.M[0]);
+    const int idx = ey * l.P + ex;
+    const unsigned sx = (unsigned)__cvta_generic_to_shared(ext + idx);
+    const unsigned syz = (unsigned)__cvta_generic_to_shared(ext + yz_plane_offset(l) + 2 * idx);
+    int slot = s0, gz = z0;
 #pragma unroll 4
-      for (int ey = 0; ey < n1; ++ey) {
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(src) : "memory");
-        sa += sstep;
-        src += row;
-      }
-      src = gplane;
-      for (int ey = n1; ey < l.EY; ++ey) {
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(src) : "memory");
-        sa += sstep;
-        src += row;
-      }
+    for (int p = pa; p < pb; ++p) {
+      const float* a = src + (size_t)gz * plane;
+      const unsigned d = 4u * (unsigned)(slot * l.Q);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sx + d), "l"(a) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(syz + 2 * d), "l"(a + Mtot) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(syz + 2 * d + 4), "l"(a + 2 * Mtot) : "memory");
+      slot = slot + 1 == l.EZ ? 0 : slot + 1;
+      gz = gz + 1 == g.M[2] ? 0 : gz + 1;
     }
   }
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
