@@ -10,7 +10,15 @@
 // (tile_z of the E_Z, with asynchronous 4-byte copies, no register round trip); a warp owns a
 // particle and its lanes own window rows; the M_G x-profiles are computed by
 // M_G lanes and broadcast into registers with warp shuffles. Per point: a 4-byte
-// load (x) and an 8-byte load (y, z interleaved) from shared memory and 8 FMA.
+// load (x) and an 8-byte load (y, z interleaved) from shared memory, and 6 FMAs with
+// torques (gather_particle; 8 with two widths or supports without a compiled variant)
+// or 5 for forces only.
+// What bounds it: shared-memory reads (12 bytes per point) and, about a quarter of the
+// time, the copy of a tile's new planes, which the other CTA of the SM covers in part.
+// 32 x 65,536 spheres on 128^3, M_G = 14, torques: 4.62 ms with 8 FMAs per point, a row
+// copied per warp and butterfly sums, 4.36 with packed sums, 4.31 with
+// full-lane copies; 8 x 65,536 rods, M_G = 12: 978, 938, 878 us; 122,231 on
+// 216^3, M_G = 10, forces only: 271 -> 245 us.
 // The pair-correction sums, when present, are added when U and W are written
 // in input order.
 #include "grid_common.cuh"

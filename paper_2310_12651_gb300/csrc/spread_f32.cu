@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(rows_threads(MGT), 1) spread_rows_kernel(Geome
 // spread_pencil_kernel (default for M_G <= 16 with 8-point tiles in x): one CTA walks a whole
 // x-pencil of binning tiles (all tiles with the same (y, z) tile index of one system; they are
 // contiguous in the tile-sorted order). Every thread owns one (y, z) row of the pencil's extended
-// (y, z) region and keeps a register row of EXT2 point pairs per component, anchored at the current
+// (y, z) region (two rows up to M_G = 12, pencil_two_rows) and keeps a register row of EXT2 point pairs per component, anchored at the current
 // half tile's x origin x0 = 4 s. The binning orders each tile's particles by the half of the tile
 // their window starts in, so the particles of half tile s, taken in order, have window starts in
 // [x0, x0 + 4): once the walk passes to half tile s + 1 the points x0 .. x0 + 3 are complete for this
