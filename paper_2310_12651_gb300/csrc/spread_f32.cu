@@ -872,7 +872,12 @@ static void pencil_variant(const Geometry<float>& g, const KernelConsts<float>& 
   const int pencils = nsys * g.ntile[1] * g.ntile[2];
   // Long pencils are split into segments when there are too few pencils for four waves of one CTA per SM
   // (thin slabs, small single systems); a segment flushes its whole register row at its end.
-  const int nseg = std::min(g.ntile[0], std::max(1, (4 * device_sm_count() + pencils - 1) / pencils));
+  int nseg = std::min(g.ntile[0], std::max(1, (4 * device_sm_count() + pencils - 1) / pencils));
+  // Two CTAs per SM empty their last waves sooner with six of those waves, as long as a segment keeps three tiles:
+  // ragged batch of 13 systems (819 pencils of 12 tiles) 340 -> 322 us, 122,231 spheres (729 of 27) 247 -> 231 us, 65,536
+  // (256 of 16) 164 -> 158 us; eight waves the same; rods in a slab (60 of 30) in two-tile segments 103 -> 113 us.
+  if constexpr (pencil_two_rows(MGT, MODE))
+    nseg = std::max(nseg, std::min(g.ntile[0] / 3, (6 * device_sm_count() + pencils - 1) / pencils));
   const int segl = (g.ntile[0] + nseg - 1) / nseg;
   const int blocks = pencils * ((g.ntile[0] + segl - 1) / segl);
   if constexpr (pencil_two_rows(MGT, MODE)) {
