@@ -228,6 +228,7 @@ void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const
   const int blocks = (n + 255) / 256;
   key_count_kernel<R><<<blocks, 256, 0, s>>>(g, n, pos, b, need);
   *launches += 1;
+  if (need == 0) return;   // no order needed (a correction that is identically zero): the position check alone
   // Every block reading all counters before its chunk costs chunks^2 / 2 chunk reads from L2: below a microsecond
   // at 16 chunks, 8 at 64 (each block's own reads are a chain of loads); past that the chunk sums pay their launch.
   const bool sums = std::max(tile_chunks, cell_chunks) > 32 && b.chunk_sum != nullptr;
