@@ -386,7 +386,16 @@ void launch_broyden_step(const R* z, const R* S, size_t m, size_t stride, int n,
 size_t tile_smem_bytes(const int tile[3], int MG);      // extended region (gather, atomic spread)
 size_t spread_smem_bytes(const int tile[3], int MG);    // whichever spread kernel the tile selects
 bool spread_uses_rows(const int tile[3], int MG);       // row-stationary spread applies
-int tile_smem_limit();
+constexpr int kTileSmemLimit = 227 * 1024;              // dynamic shared memory of a block without static shared memory
+inline int tile_smem_limit() { return kTileSmemLimit; }
+// Lets kernel k be launched with up to `most` bytes of dynamic shared memory. The limit belongs to the kernel in the
+// context, not to a handle, and a launch above it is refused, so every caller passes the same value for one kernel, the
+// largest any handle can need: with a size of the handle's own, a thread that works with a smaller handle could lower
+// the limit between another thread's call here and its launch. The occupancy follows the launch's own size.
+template <typename K>
+inline void allow_dynamic_smem(K* k, size_t most) {
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 // spread_kernel: 0 = choose, 1 = row-stationary, 2 = shared atomics, 3 = tensor cores where eligible
 // (fcm_params.spread_kernel).
 void launch_spread_f32(const Geometry<float>& g, const KernelConsts<float>& kc, bool torque, int spread_kernel,

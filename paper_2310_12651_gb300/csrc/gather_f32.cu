@@ -414,7 +414,7 @@ static void gather_variant(const Geometry<float>& g, const KernelConsts<float>& 
                            cudaStream_t s) {
   const size_t smem = tile_smem_bytes(g.tile, g.MG);
   auto k = gather_tile_kernel<MGT, GUARD, TORQUE, SAMEW>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k, kTileSmemLimit);   // any tile and support
   const int nsys = g.nsys > 1 ? g.nsys : 1;
   const int pencils = nsys * g.ntile[0] * g.ntile[1];
   // one CTA per z-pencil of tiles; pencils are split into segments when there are too few of them for

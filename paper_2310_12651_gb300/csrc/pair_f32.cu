@@ -460,7 +460,7 @@ static void cluster_variant(const Geometry<float>& g, const PairConsts<float>& p
                             const PairPoly& poly, const BinBuffers& b, cudaStream_t s) {
   const size_t smem = cluster_smem<TORQUE, WARPS>();
   auto k = pair_cluster_kernel<TORQUE, SHIFT, WARPS>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k, smem);
   k<<<b.ncells, WARPS * 32, smem, s>>>(g, pc, tab, poly, (const float4*)b.c_pos, (const float4*)b.c_F,
                                        (const float4*)b.c_T, b.cell_start, (float4*)b.c_sum);
 }

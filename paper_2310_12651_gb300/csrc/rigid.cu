@@ -547,9 +547,10 @@ void launch_rigid_residual(const R* V, const R* x, const R* ft, const R* arm, co
 template <typename R>
 void launch_body_precond(const R* arm, const int* body_off, int nb, int kmax, const double L[3], double a, double eta,
                          R* aT, int* flags, cudaStream_t s, long long* launches) {
+  auto bytes = [](int k) { const size_t m = 3 * (size_t)k + 6; return sizeof(R) * (m * m + m); };
   const int m = 3 * kmax + 6;
-  const size_t smem = sizeof(R) * ((size_t)m * m + m);
-  cudaFuncSetAttribute(body_precond_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = bytes(kmax);
+  allow_dynamic_smem(body_precond_kernel<R>, bytes(kRigidBodyMax));
   body_precond_kernel<R><<<nb, 256, smem, s>>>(arm, body_off, nb, L[0], L[1], L[2], a, eta, m, aT, flags);
   *launches += 1;
 }

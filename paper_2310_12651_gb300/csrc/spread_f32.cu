@@ -833,8 +833,6 @@ size_t tile_smem_bytes(const int tile[3], int MG) {
   return sizeof(float) * (3 * (size_t)l.C + 1);   // + 1: the gather's (y, z) plane starts 8-byte aligned
 }
 
-int tile_smem_limit() { return 227 * 1024; }
-
 static int rows_mgt(int MG) {
   switch (MG) {
     case 10: case 12: case 14: case 16: return MG;
@@ -860,7 +858,7 @@ static void pencil_launch(const Geometry<float>& g, const KernelConsts<float>& k
   const int rows = (g.tile[1] + g.MG - 1) * (g.tile[2] + g.MG - 1);
   const int threads = (((rows + R - 1) / R + 31) / 32) * 32;
   auto k = spread_pencil_kernel<MGT, GUARD, MODE, R>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k, smem);
   k<<<blocks, threads, smem, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F, (const float4*)b.t_T,
                                   b.tile_start, grid, segl);
 }
@@ -910,11 +908,11 @@ static void rows_variant(const Geometry<float>& g, const KernelConsts<float>& kc
     const int nsys = g.nsys > 1 ? g.nsys : 1;
     const int blocks = nsys * ((g.ntile[0] + 1) / 2) * g.ntile[1] * g.ntile[2];
     auto k = spread_rows_kernel<MGT, GUARD, TORQUE, SAMEW, 16>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem(k, smem);
     k<<<blocks, threads, smem, s>>>(g, kc, pos, F, T, b.tile_start, grid);
   } else {
     auto k = spread_rows_kernel<MGT, GUARD, TORQUE, SAMEW, 8>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem(k, smem);
     k<<<b.ntiles, threads, smem, s>>>(g, kc, pos, F, T, b.tile_start, grid);
   }
 }
@@ -924,7 +922,7 @@ static void atomic_variant(const Geometry<float>& g, const KernelConsts<float>& 
                            float* grid, cudaStream_t s) {
   const size_t smem = tile_smem_bytes(g.tile, g.MG);
   auto k = spread_tile_kernel<MGT, GUARD, TORQUE, SAMEW>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k, kTileSmemLimit);   // any tile and support
   k<<<b.ntiles, 256, smem, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F, (const float4*)b.t_T,
                                 b.tile_start, grid);
 }

@@ -324,7 +324,7 @@ void mma_variant(const Geometry<float>& g, const KernelConsts<float>& kc, const 
   const int nsys = g.nsys > 1 ? g.nsys : 1;
   const int blocks = nsys * ((g.ntile[0] + 1) / 2) * g.ntile[1] * g.ntile[2];
   auto k = spread_mma_kernel<MGT, TORQUE, SAMEW>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+  allow_dynamic_smem(k, S::SMEM);
   k<<<blocks, kMmaThreads, S::SMEM, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F,
                                          (const float4*)b.t_T, b.tile_start, grid, b.status);
 }

@@ -422,7 +422,7 @@ void tc_variant(const Geometry<float>& g, const KernelConsts<float>& kc, const B
   const int blocks = nsys * g.ntile[1] * g.ntile[2];
   const int threads = 32 * (S::NPW + 1);   // producer warps + the issuer warp
   auto k = spread_pencil_tc_kernel<MGT, TORQUE>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+  allow_dynamic_smem(k, S::SMEM);
   k<<<blocks, threads, S::SMEM, s>>>(g, kc, (const float4*)b.t_pos, (const float4*)b.t_F,
                                         (const float4*)b.t_T, b.tile_start, grid, b.status);
 }

@@ -26,6 +26,7 @@ constexpr int kZThreads = 192;   // a multiple of three components times the col
 // two copies within 50 KB (25 KB in FP64), so that short columns still give every thread a butterfly (16 points: 19 -> 9
 // us on a 240 x 240 x 16 grid); fewer again where that leaves less than two blocks per SM.
 constexpr size_t kBlockSmem = 50 * 1024;
+constexpr size_t kPlanSmem = kTileSmemLimit / 2 - 1024;   // the most a plan may take: two blocks per SM
 
 template <typename R> struct Pair2;
 template <> struct Pair2<float> { typedef float2 T; };
@@ -288,7 +289,7 @@ bool make_zplan(int N, bool fp64, ZPlan* p) {
   p->steps = 0;
   // two blocks per SM at least: one reads or writes global memory while the other works in shared memory
   p->lines_log2 = fp64 ? 2 : 3;
-  if (N < 2 || z_smem(N, p->lines_log2, fp64) > (size_t)tile_smem_limit() / 2 - 1024) return false;
+  if (N < 2 || z_smem(N, p->lines_log2, fp64) > kPlanSmem) return false;
   while (p->lines_log2 < 6 && z_smem(N, p->lines_log2 + 1, fp64) <= (fp64 ? kBlockSmem / 2 : kBlockSmem)) p->lines_log2 += 1;
   // the fewest steps, then the smallest largest radix (every step is a pass over shared memory; a radix is registers)
   static const int kRadix[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 16};
@@ -344,7 +345,7 @@ void launch_zsolve(const Geometry<R>& g, const ZPlan& plan, R eta, R factor, con
   const size_t smem = z_smem(p.N, p.lines_log2, sizeof(R) == 8);
   typedef typename Pair2<R>::T T2;
   auto k = factor == R(0) ? zsolve_kernel<R, false> : zsolve_kernel<R, true>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k, kPlanSmem);
   k<<<grid, kZThreads, smem, s>>>(p, g.M[0], g.M[1], kx0, ky0, kz0, scale, (const T2*)table, (T2*)spectrum);
   *launches += 1;
 }
