@@ -198,11 +198,16 @@ void build_pair_table(const PairConsts<double>& pd, double r_lo, double r_hi, in
 // The fit of PairPoly: for each coefficient f the weights w = exp(-r^2 / 4 Sigma^2) r^d / scale turn the error into
 // one relative to the self mobility of its block (bt and dl act with r^2, cr with r), and a polynomial in t (affine
 // in 1/r, Chebyshev basis) is fitted by iteratively reweighted least squares, whose weights tend to the minimax
-// solution. False unless all five errors, with the coefficients rounded to FP32, are below kPairPolyTol.
-constexpr double kPairPolyTol = 6e-9;   // 146 neighbours add up to 7e-8 of the self mobility at random
+// solution. It holds if every error is below the tolerance plus the rounding of an evaluation in FP32 as the kernel's
+// (kPairPolyRound of the value), at twice as many radii as the fit used, none of them its own.
+// The tolerance keeps the error of every function over the pairs within r_c at or below that of the cubic table
+// (volume-weighted rms, nine parameter sets; Sigma = 1.6, r_c = 7.2 Sigma: al 1.26e-9 of the self mobility by the table,
+// 0.9e-9 here, 3.6e-9 with degree 9 and a tolerance of 6e-9; al decays slowest and needs degree 11 at the same r_near).
+constexpr double kPairPolyTol = 1e-9;
+constexpr double kPairPolyRound = 1e-6;
 
 static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn, double r_c, PairPoly* out) {
-  constexpr int D = kPairPolyDegree, N = 48;
+  constexpr int DM = kPairPolyDegree, N = 48, NV = 2 * N;
   PairConsts<double> pc = pd;
   pc.rs2 = 0.0;
   const double e4 = 1.0 / (4.0 * pd.Sg2);
@@ -210,32 +215,40 @@ static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn
   const double scale[5] = {vf, vf, std::sqrt(vf * wt), wt, wt};
   const int power[5] = {0, 2, 1, 0, 2};
   const double alpha = 2.0 / (1.0 / rn - 1.0 / r_c), beta = 1.0 - alpha / rn;
-  double T[N][D + 1], f[5][N], w[5][N];
+  out->scale = (float)alpha;
+  out->offset = (float)beta;
+  out->expo = (float)(-e4 * 1.4426950408889634);
+  out->near2 = (float)(rn * rn);
+  // the five functions at r, in units of their self mobilities, and those units
+  auto values = [&](double r, double (&f)[5], double (&u)[5]) {
+    pair_coeffs<double>(r * r, pc, f[0], f[1], f[2], f[3], f[4]);
+    for (int q = 0; q < 5; ++q) {
+      u[q] = (power[q] == 0 ? 1.0 : (power[q] == 1 ? r : r * r)) / scale[q];
+      f[q] *= u[q];
+    }
+  };
+  double T[N][DM + 1], f[N][5], w[N][5];
   for (int k = 0; k < N; ++k) {
     const double t = std::cos(kPi * (k + 0.5) / N), r = alpha / (t - beta);
-    double c[5];
-    pair_coeffs<double>(r * r, pc, c[0], c[1], c[2], c[3], c[4]);
-    for (int q = 0; q < 5; ++q) {
-      const double u = (power[q] == 0 ? 1.0 : (power[q] == 1 ? r : r * r)) / scale[q];
-      f[q][k] = c[q] * u;
-      w[q][k] = std::exp(-r * r * e4) * u;
-    }
+    values(r, f[k], w[k]);
+    for (int q = 0; q < 5; ++q) w[k][q] *= std::exp(-r * r * e4);
     T[k][0] = 1.0;
     T[k][1] = t;
-    for (int m = 2; m <= D; ++m) T[k][m] = 2.0 * t * T[k][m - 1] - T[k][m - 2];
+    for (int m = 2; m <= DM; ++m) T[k][m] = 2.0 * t * T[k][m - 1] - T[k][m - 2];
   }
-  double tm[D + 1][D + 1] = {};   // powers of t of the Chebyshev polynomials
+  double tm[DM + 1][DM + 1] = {};   // powers of t of the Chebyshev polynomials
   tm[0][0] = 1.0;
   tm[1][1] = 1.0;
-  for (int m = 2; m <= D; ++m)
-    for (int j = 0; j <= D; ++j) tm[m][j] = (j > 0 ? 2.0 * tm[m - 1][j - 1] : 0.0) - tm[m - 2][j];
+  for (int m = 2; m <= DM; ++m)
+    for (int j = 0; j <= DM; ++j) tm[m][j] = (j > 0 ? 2.0 * tm[m - 1][j - 1] : 0.0) - tm[m - 2][j];
   for (int q = 0; q < 5; ++q) {
-    double lw[N], x[D + 1] = {};
+    const int D = pair_poly_degree(q);
+    double lw[N], x[DM + 1] = {};
     for (int k = 0; k < N; ++k) lw[k] = 1.0;
     for (int it = 0; it < 8; ++it) {
-      double A[D + 1][D + 2] = {};
+      double A[DM + 1][DM + 2] = {};   // the right-hand side in column D + 1
       for (int k = 0; k < N; ++k) {
-        const double ww = lw[k] * w[q][k] * w[q][k], wf = lw[k] * w[q][k] * f[q][k];
+        const double ww = lw[k] * w[k][q] * w[k][q], wf = lw[k] * w[k][q] * f[k][q];
         for (int i = 0; i <= D; ++i) {
           for (int j = 0; j <= i; ++j) A[i][j] += ww * T[k][i] * T[k][j];
           A[i][D + 1] += wf * T[k][i];
@@ -262,7 +275,7 @@ static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn
       for (int k = 0; k < N; ++k) {
         double s = 0.0;
         for (int m = 0; m <= D; ++m) s += x[m] * T[k][m];
-        err[k] = std::fabs(w[q][k] * s - f[q][k]);
+        err[k] = std::fabs(w[k][q] * s - f[k][q]);
         worst = std::max(worst, err[k]);
       }
       if (!(worst > 0.25 * kPairPolyTol)) break;   // good enough
@@ -273,16 +286,20 @@ static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn
       for (int m = j; m <= D; ++m) s += x[m] * tm[m][j];
       out->c[q][j] = (float)s;
     }
-    for (int k = 0; k < N; ++k) {
-      double s = 0.0;
-      for (int j = D; j >= 0; --j) s = s * T[k][1] + (double)out->c[q][j];
-      if (!(std::fabs(w[q][k] * s - f[q][k]) < kPairPolyTol)) return false;
+  }
+  for (int k = 0; k < NV; ++k) {
+    const double t = std::cos(kPi * (k + 0.5) / NV);
+    const float r2 = (float)std::pow(alpha / (t - beta), 2.0);
+    double fr[5], u[5];
+    values(std::sqrt((double)r2), fr, u);
+    const float tf = std::fma((float)(1.0 / std::sqrt((double)r2)), out->scale, out->offset), e = std::exp2(r2 * out->expo);
+    for (int q = 0; q < 5; ++q) {
+      const int D = pair_poly_degree(q);
+      float s = out->c[q][D];
+      for (int j = D - 1; j >= 0; --j) s = std::fma(s, tf, out->c[q][j]);
+      if (!(std::fabs(u[q] * (double)(e * s) - fr[q]) < kPairPolyTol + kPairPolyRound * std::fabs(fr[q]))) return false;
     }
   }
-  out->scale = (float)alpha;
-  out->offset = (float)beta;
-  out->expo = (float)(-e4 * 1.4426950408889634);
-  out->near2 = (float)(rn * rn);
   out->ok = 1;
   return true;
 }

@@ -250,9 +250,11 @@ __device__ inline void pair_coeffs_table(float r2, const PairConsts<float>& C, c
 }
 
 // FP32 coefficients beyond r_near (pair_f32.cu): c[f] holds function f (al, bt, cr, gm, dl) as
-// exp2(r^2 expo) sum_m c[f][m] t^m with t = scale / r + offset in [-1, 1] on [r_near, r_c]; near2 = r_near^2.
+// exp2(r^2 expo) sum_m c[f][m] t^m, m <= pair_poly_degree(f), with t = scale / r + offset in [-1, 1] on [r_near, r_c];
+// near2 = r_near^2.
 // ok == 0: no such fit, every pair uses the table.
-constexpr int kPairPolyDegree = 9;
+constexpr int kPairPolyDegree = 11;   // the largest of the five
+__host__ __device__ constexpr int pair_poly_degree(int f) { return f == 0 ? kPairPolyDegree : 9; }
 struct PairPoly {
   float c[5][kPairPolyDegree + 1];
   float scale, offset, expo, near2;

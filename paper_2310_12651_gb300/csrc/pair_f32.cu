@@ -15,10 +15,10 @@
 //   close together). Lanes test 32 candidates against all four; candidates within r_c of any are queued, and a
 //   pass of 32 queued partners evaluates 4 x 32 pairs from registers. At 5% (146 neighbours) 61% of those are
 //   within r_c; one load of the partner and one addition of its sums serve four pairs;
-// * beyond a radius r_near the coefficients are exp(-r^2 / 4 Sigma^2) times polynomials of degree 9 in 1/r,
-//   fitted to the closed form in FP64 when the handle is made (weighted minimax, error below 6e-9 of the
-//   self mobility; r_near is the smallest radius at which the fit reaches that, 2.1 to 3.2 Sigma): 45 FMAs with
-//   constant operands instead of 20 random 16-byte reads per quarter warp;
+// * beyond a radius r_near the coefficients are exp(-r^2 / 4 Sigma^2) times polynomials in 1/r (degree 11 for al, 9 for
+//   the others), fitted to the closed form in FP64 when the handle is made (weighted minimax, error below 1e-9 of
+//   the self mobility and FP32 rounding; r_near is the smallest radius at which the fit reaches that, 2.1 to 3.0
+//   Sigma): 47 FMAs with constant operands instead of 20 random 16-byte reads per quarter warp;
 // * closer pairs (5%) go to a second queue, evaluated with the piecewise-cubic table (Taylor series below
 //   sigma/2, which covers coincident points). Where no such fit exists (r_near above 0.6 r_c, Sigma_D far from
 //   Sigma) and in cells that see a load that is not finite (or above 1e18), whose product with a masked pair's zero is NaN,
@@ -65,10 +65,12 @@ __device__ __forceinline__ void red4(float4* p, float a, float b, float c) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(0.f) : "memory");
 }
 
-__device__ __forceinline__ float poly_eval(const float (&c)[kPairPolyDegree + 1], float t) {
-  float s = c[kPairPolyDegree];
+template <int F>
+__device__ __forceinline__ float poly_eval(const PairPoly& p, float t) {
+  constexpr int D = pair_poly_degree(F);
+  float s = p.c[F][D];
 #pragma unroll
-  for (int m = kPairPolyDegree - 1; m >= 0; --m) s = fmaf(s, t, c[m]);
+  for (int m = D - 1; m >= 0; --m) s = fmaf(s, t, p.c[F][m]);
   return s;
 }
 
@@ -303,8 +305,8 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
               const float t0 = fmaf(ir.x, poly.scale, poly.offset), t1 = fmaf(ir.y, poly.scale, poly.offset);
               const float2 e = make_float2(hit0 && !close0 ? exp2_approx(r2.x * poly.expo) : 0.f,
                                            hit1 && !close1 ? exp2_approx(r2.y * poly.expo) : 0.f);
-              const float2 al = mul2(e, make_float2(poly_eval(poly.c[0], t0), poly_eval(poly.c[0], t1)));
-              const float2 bt = mul2(e, make_float2(poly_eval(poly.c[1], t0), poly_eval(poly.c[1], t1)));
+              const float2 al = mul2(e, make_float2(poly_eval<0>(poly, t0), poly_eval<0>(poly, t1)));
+              const float2 bt = mul2(e, make_float2(poly_eval<1>(poly, t0), poly_eval<1>(poly, t1)));
               const float2 Fx = si[h * W2 + 3], Fy = si[h * W2 + 4], Fz = si[h * W2 + 5];
               const float2 bj = mul2(bt, dot2(dx, dy, dz, two(Fj.x), two(Fj.y), two(Fj.z)));
               const float2 bi = mul2(bt, dot2(dx, dy, dz, Fx, Fy, Fz));
@@ -315,9 +317,9 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
               v[1] = fma2(al, Fy, fma2(bi, dy, v[1]));
               v[2] = fma2(al, Fz, fma2(bi, dz, v[2]));
               if constexpr (TORQUE) {
-                const float2 cr = mul2(e, make_float2(poly_eval(poly.c[2], t0), poly_eval(poly.c[2], t1)));
-                const float2 gm = mul2(e, make_float2(poly_eval(poly.c[3], t0), poly_eval(poly.c[3], t1)));
-                const float2 dl = mul2(e, make_float2(poly_eval(poly.c[4], t0), poly_eval(poly.c[4], t1)));
+                const float2 cr = mul2(e, make_float2(poly_eval<2>(poly, t0), poly_eval<2>(poly, t1)));
+                const float2 gm = mul2(e, make_float2(poly_eval<3>(poly, t0), poly_eval<3>(poly, t1)));
+                const float2 dl = mul2(e, make_float2(poly_eval<4>(poly, t0), poly_eval<4>(poly, t1)));
                 const float2 nr = make_float2(-cr.x, -cr.y);
                 const float2 cx = mul2(cr, dx), cy = mul2(cr, dy), cz = mul2(cr, dz);
                 const float2 nx = mul2(nr, dx), ny = mul2(nr, dy), nz = mul2(nr, dz);
