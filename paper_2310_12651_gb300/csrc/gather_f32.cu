@@ -191,13 +191,17 @@ __device__ __forceinline__ void gather_particle(const Geometry<float>& g, const 
 // CTAs per SM asked of the compiler: what the region's shared memory allows. Forces only with M_G = 10, three
 // (122,231 spheres on 216^3: 271 us, with two 312 us), with smaller supports more; from M_G = 12 on, and with
 // torques, two of 128 registers a thread (one of more registers: 32 x 65,536 spheres, M_G = 14, 5.76 against
-// 4.36 ms); the two largest supports' regions leave one.
-constexpr int gather_ctas(int MGT, bool guard, bool torque) {
-  return MGT > 16 ? 1 : (torque || (!guard && MGT >= 12) ? 2 : (MGT <= 8 ? 4 : 3));
+// 4.36 ms). Supports up to 8 with torques and one width fit three (40,000 spheres on 72^3, M_G = 8: 51 us, with two
+// 62 us); of the two largest, whose regions are made to leave two, M_G up to 20 with one width takes them (M_G = 18 /
+// 20: 372 / 1,198 us, with one 521 / 2,010 us), the others are no faster so (M_G = 24: 1,472 us, with two 1,529 us).
+constexpr int gather_ctas(int MGT, bool guard, bool torque, bool samew) {
+  if (MGT > 16) return MGT <= 20 && samew ? 2 : 1;
+  if (MGT <= 8) return !torque ? 4 : (samew ? 3 : 2);
+  return torque || (!guard && MGT >= 12) ? 2 : 3;
 }
 
 template <int MGT, bool GUARD, bool TORQUE, bool SAMEW>
-__global__ void __launch_bounds__(256, gather_ctas(MGT, GUARD, TORQUE)) gather_tile_kernel(Geometry<float> g, KernelConsts<float> kc,
+__global__ void __launch_bounds__(256, gather_ctas(MGT, GUARD, TORQUE, SAMEW)) gather_tile_kernel(Geometry<float> g, KernelConsts<float> kc,
                                                           const float4* __restrict__ pos,
                                                           const int* __restrict__ tstart,
                                                           const float* __restrict__ grid,
