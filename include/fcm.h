@@ -411,7 +411,7 @@ int fcm_server_destroy(fcm_server* s);
  *            per dimension, must number at most FCM_NOALLOC_MAX_CELLS
  *   pos, F, T (T may be NULL), U, W (W may be NULL): as for fcm_apply, on the
  *            current CUDA device
- * It allocates nothing: all scratch (about 6.4 MB) is one fixed file-scope
+ * It allocates nothing: all scratch (about 9.6 MB) is one fixed file-scope
  * device array, held by every CUDA context that loads the library's device
  * code (normally one per GPU) until the process exits. With lazy module
  * loading the context reserves it at the first call made in it: make that

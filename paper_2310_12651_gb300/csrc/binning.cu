@@ -29,6 +29,7 @@ template <typename R>
 __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, const R* __restrict__ pos,
                                                         BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && (need & kBinCells) && b.crowd) b.crowd[1] = 0;   // for the scan to fill
   if (b.n_dev) n = min(n, *b.n_dev);
   if (i >= n) return;
   const int sys = system_of(b, i);
@@ -108,6 +109,17 @@ __global__ void __launch_bounds__(kScanThreads) chunk_sum_kernel(BinBuffers b, i
   }
 }
 
+// Lists a pair cell's parts if it is crowded.
+__device__ inline void note_cell(const BinBuffers& b, int cell, int count) {
+  if (count <= kCrowdCell) return;
+  const int parts = crowd_parts(count);
+  int* item = b.crowd + 2 + 2 * atomicAdd(&b.crowd[1], parts);
+  for (int p = 0; p < parts; ++p, item += 2) {
+    item[0] = cell;
+    item[1] = p;
+  }
+}
+
 // Exclusive scan: block (c, s) writes the starts of chunk c of system s's bins. It adds up the counters
 // before its chunk by itself (from the chunk sums when they were made), so the blocks need no order. A system's
 // bins are contiguous and its particles are the stacked rows from sys_off[s]: segments start there.
@@ -131,6 +143,17 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(BinBuffers b, int ti
   for (int k = 0; k < kPer; ++k) {
     v[k] = first + k < p.nb ? p.count[first + k] : 0;
     own += v[k];
+  }
+  if (!p.tiles && b.crowd) {
+    const int at = (int)blockIdx.y * p.nb + first;   // the thread's first counter
+    static_assert(kPer == 4, "two neighbouring threads per cell of eight counters");
+    if (b.cell_parts == 8) {
+      const int cell = own + __shfl_xor_sync(0xffffffffu, own, 1);
+      if (!(lane & 1)) note_cell(b, at / 8, cell);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) note_cell(b, at + k, v[k]);
+    }
   }
   before = warp_total(before);
   int incl = own;
@@ -211,6 +234,8 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
       const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
       ((float4*)b.c_sum)[2 * (size_t)dc] = zero;
       ((float4*)b.c_sum)[2 * (size_t)dc + 1] = zero;
+      if (b.crowd[1] > 0)
+        for (int k = 0; k < 3; ++k) reinterpret_cast<float4*>(b.c_sum64 + 6 * (size_t)dc)[k] = zero;
     }
     ((Vec4<R>*)b.c_pos)[dc] = p;
     ((Vec4<R>*)b.c_F)[dc] = f;

@@ -25,7 +25,15 @@
 //   every pair goes that way;
 // * partners' sums are added to per-particle accumulators in cell order with 16-byte reductions in L2 (one for
 //   U, one for W: a reduction costs the same for one float or four), the cluster's sums after a halving
-//   reduction across lanes; a small kernel brings them to input order. The order of the additions is not fixed.
+//   reduction across lanes; a small kernel brings them to input order. The order of the additions is not fixed;
+// * a cell of more than kCrowdCell particles is crowded: it is listed in parts by the binning's scan, which the last CTAs
+//   of the launch share out when they have done their own cells, and its sums are reduced in FP64, six reductions instead
+//   of two. A particle receives one addition per cluster that meets it. The 30 of a suspension (5%, 146 neighbours) cost
+//   less than the coefficients' rounding; hundreds of them do not, and FP64 throughout costs all others 10%. Error of U's
+//   pair part against 64 bits (rms, of 1e-9) with one FP32 sum per chunk of candidates and cell, compensated for a
+//   particle's own pairs / FP32 reductions alone / FP64 in crowded cells: 65,536 at 5% 190 / 188 / 185, 20,000 with 640
+//   neighbours 245 / 282 / 216, 4,000 in one cell 149 / 203 / 146. Sharing out keeps a suspension that fills a corner
+//   of its box from running in a few CTAs: 65,536 in 125 cells 2.76 / 3.58 / 0.69 ms, 4,000 in one cell 11.9 / 9.3 / 0.21 ms.
 // Measured against one particle at a time, tables and shared-memory atomics: 32 systems of 65,536 at 5%, torques,
 // 4.04 -> 2.93 ms; 1,048,576 at 10% 2.64 -> 1.84 ms; 122,231 at 0.8%, forces only, 153 -> 95 us. Now 1,020
 // instructions per particle, the schedulers issue 58% of the time and the FMA pipe is busy 45%.
@@ -42,8 +50,9 @@ constexpr int kCluster = 4;
 constexpr int kQueue = 64;                      // fewer than 32 left over, 32 of a pass
 constexpr int kNearQueue = 32 + 32 * kCluster;  // fewer than 32 left over, all pairs of a pass
 
-// CTAs per SM that the register file is split for, by warps of a CTA and by the sums a thread keeps.
-__host__ __device__ constexpr int cell_blocks(int warps, bool torque) { return warps == 2 || !torque ? 6 : 4; }
+// CTAs per SM that the register file is split for, by warps of a CTA and by the sums a thread keeps (128 registers, 80 for
+// four warps without torques); the shared memory leaves six of two warps with torques.
+__host__ __device__ constexpr int cell_blocks(int warps, bool torque) { return warps == 2 ? 8 : (torque ? 4 : 6); }
 
 template <bool TORQUE, int WARPS>
 constexpr size_t cluster_smem() {
@@ -63,6 +72,19 @@ __device__ inline bool bounded3(float4 v) { return fabsf(v.x) < 1e18f && fabsf(v
 
 __device__ __forceinline__ void red4(float4* p, float a, float b, float c) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(0.f) : "memory");
+}
+
+// Three sums to the accumulators of particle k, U's (w = 0) or W's (w = 1).
+template <bool CROWDED>
+__device__ __forceinline__ void add_sums(float4* psum, double* psum64, int k, int w, float a, float b, float c) {
+  if (CROWDED) {
+    double* q = psum64 + 6 * (size_t)k + 3 * w;
+    atomicAdd(q, (double)a);
+    atomicAdd(q + 1, (double)b);
+    atomicAdd(q + 2, (double)c);
+  } else {
+    red4(psum + 2 * (size_t)k + w, a, b, c);
+  }
 }
 
 template <int F>
@@ -108,20 +130,22 @@ __device__ __forceinline__ float2 dot2(float2 ax, float2 ay, float2 az, float2 b
 
 }  // namespace
 
-template <bool TORQUE, bool SHIFT, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
-    pair_cluster_kernel(Geometry<float> g, PairConsts<float> pc, PairTable tab, PairPoly poly,
-                        const float4* __restrict__ cpos, const float4* __restrict__ cF, const float4* __restrict__ cT,
-                        const int* __restrict__ cstart, float4* __restrict__ psum) {
+// The pairs of a cell's particles with themselves and with the half shell: of all of them, or of a crowded cell's clusters
+// of one part (every crowd_parts-th WARPS of them).
+template <bool TORQUE, bool SHIFT, int WARPS, bool CROWDED>
+__device__ __forceinline__ void cell_pairs(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab,
+                                           const PairPoly& poly, const float4* __restrict__ cpos,
+                                           const float4* __restrict__ cF, const float4* __restrict__ cT,
+                                           const int* __restrict__ cstart, float4* __restrict__ psum,
+                                           double* __restrict__ psum64, int cell, int part) {
   constexpr int V = TORQUE ? 6 : 3;   // sums per particle
   constexpr int W2 = TORQUE ? 9 : 6;  // values per particle of a cluster: position, force, torque
   extern __shared__ float4 sm4[];
   float4* spos = sm4;                 // position from the cell's corner; w: r_c^2 (with margin) - |position|^2
   float4* sF = spos + kHalfChunk;
   float4* sT = sF + kHalfChunk;
-  const int cell = blockIdx.x;
   const int i_begin = cstart[cell], i_end = cstart[cell + 1];
-  if (i_begin >= i_end) return;
+  if (i_begin >= i_end || (!CROWDED && i_end - i_begin > kCrowdCell)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float4* si_all = TORQUE ? sT + kHalfChunk : sT;                     // [warps][2 pairs][value] float2, padded
   float4* pshift = si_all + 3 * kCluster * WARPS;
@@ -138,7 +162,7 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
   __syncthreads();
   const int total = meta[2 * kPieces + 1];
   const unsigned lt = (1u << lane) - 1u;
-  const int ni = i_end - i_begin;
+  const int ni = i_end - i_begin, parts = CROWDED ? crowd_parts(ni) : 1;
   // Positions are staged from a point beside the cell's first particle: small numbers, so the test can use
   // |x_i|^2 + |x_j|^2 - 2 x_i.x_j (three FMAs per particle) with a margin for its cancellation (at most 20
   // roundings of 2^-24 of the squared extent of two cells). The point is a multiple of the box edge's last place, so
@@ -189,7 +213,7 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
     __syncthreads();
     const bool all_near = *odd_load != 0;
 
-    for (int cl = warp; kCluster * cl < ni; cl += WARPS) {
+    for (int cl = warp + WARPS * part; kCluster * cl < ni; cl += WARPS * parts) {
       const int a = kCluster * cl;              // first particle of the cluster (slot of the own cell)
       const int ci = min(kCluster, ni - a);
       const int first = max(a + 1 - cb, 0);     // candidates after the first particle's own slot
@@ -343,9 +367,10 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
               }
             }
             if (on) {
-              float4* o = psum + 2 * (size_t)sidx[k];
-              red4(o, v[0].x + v[0].y, v[1].x + v[1].y, v[2].x + v[2].y);
-              if constexpr (TORQUE) red4(o + 1, v[3].x + v[3].y, v[4].x + v[4].y, v[5].x + v[5].y);
+              const int o = sidx[k];
+              add_sums<CROWDED>(psum, psum64, o, 0, v[0].x + v[0].y, v[1].x + v[1].y, v[2].x + v[2].y);
+              if constexpr (TORQUE)
+                add_sums<CROWDED>(psum, psum64, o, 1, v[3].x + v[3].y, v[4].x + v[4].y, v[5].x + v[5].y);
             }
           }
           while (near) {   // few lanes have any
@@ -389,9 +414,9 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
               v[4] = fmaf(ei, dy, gm * Ti.y) - (Fi.z * cx - Fi.x * cz);
               v[5] = fmaf(ei, dz, gm * Ti.z) - (Fi.x * cy - Fi.y * cx);
             }
-            float4* o = psum + 2 * (size_t)sidx[k];
-            red4(o, v[0], v[1], v[2]);
-            if constexpr (TORQUE) red4(o + 1, v[3], v[4], v[5]);
+            const int o = sidx[k];
+            add_sums<CROWDED>(psum, psum64, o, 0, v[0], v[1], v[2]);
+            if constexpr (TORQUE) add_sums<CROWDED>(psum, psum64, o, 1, v[3], v[4], v[5]);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -428,15 +453,37 @@ __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
 #pragma unroll
         for (int c = 0; c < 3; ++c) sum[c] += __shfl_xor_sync(kFullMask, sum[c], o);
       const int m = 2 * (lane >> 4) + ((lane >> 3) & 1), w = TORQUE ? (lane >> 2) & 1 : 0;
-      if ((lane & (TORQUE ? 3 : 7)) == 0 && m < ci) red4(psum + 2 * (size_t)(i_begin + a + m) + w, sum[0], sum[1], sum[2]);
+      if ((lane & (TORQUE ? 3 : 7)) == 0 && m < ci)
+        add_sums<CROWDED>(psum, psum64, i_begin + a + m, w, sum[0], sum[1], sum[2]);
       __syncwarp();
     }
+  }
+}
+
+// CTA c takes cell c unless it is crowded. The last `sharers` CTAs (as many as run at once; more of them than cells where
+// cells are few) then share the crowded cells' parts.
+template <bool TORQUE, bool SHIFT, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
+    pair_cluster_kernel(Geometry<float> g, PairConsts<float> pc, PairTable tab, PairPoly poly,
+                        const float4* __restrict__ cpos, const float4* __restrict__ cF, const float4* __restrict__ cT,
+                        const int* __restrict__ cstart, float4* __restrict__ psum, double* __restrict__ psum64,
+                        const int* __restrict__ crowd, int ncells, int sharers) {
+  if ((int)blockIdx.x < ncells)
+    cell_pairs<TORQUE, SHIFT, WARPS, false>(g, pc, tab, poly, cpos, cF, cT, cstart, psum, psum64, blockIdx.x, 0);
+  int k = (int)blockIdx.x - ((int)gridDim.x - sharers);
+  if (k < 0) return;
+  for (const int items = crowd[1]; k < items; k += sharers) {
+    __syncthreads();   // the next part reuses the shared memory
+    cell_pairs<TORQUE, SHIFT, WARPS, true>(g, pc, tab, poly, cpos, cF, cT, cstart, psum, psum64, crowd[2 + 2 * k],
+                                           crowd[3 + 2 * k]);
   }
 }
 
 // Pair sums in cell order, plus the self terms, to input order: U = or U += (ADD), W likewise.
 template <bool ADD>
 __global__ void __launch_bounds__(256) pair_merge_kernel(PairConsts<float> pc, const float4* __restrict__ psum,
+                                                         const double* __restrict__ psum64,
+                                                         const int* __restrict__ crowd,
                                                          const float4* __restrict__ cF, const float4* __restrict__ cT,
                                                          const unsigned* __restrict__ slot, int n,
                                                          const int* __restrict__ n_dev, float* __restrict__ U,
@@ -445,12 +492,18 @@ __global__ void __launch_bounds__(256) pair_merge_kernel(PairConsts<float> pc, c
   if (n_dev) n = min(n, *n_dev);
   if (i >= n) return;
   const size_t s = slot[i], o = 3 * (size_t)i;
-  const float4 a = psum[2 * s], F = cF[s];
+  const float4 F = cF[s];
+  float4 a = psum[2 * s], b = psum[2 * s + 1];   // all loads before the branch
+  if (crowd[1] > 0) {   // some sums are in FP64
+    const double* q = psum64 + 6 * s;
+    a = make_float4((float)(a.x + q[0]), (float)(a.y + q[1]), (float)(a.z + q[2]), 0.f);
+    b = make_float4((float)(b.x + q[3]), (float)(b.y + q[4]), (float)(b.z + q[5]), 0.f);
+  }
   const float u[3] = {fmaf(pc.selfVF, F.x, a.x), fmaf(pc.selfVF, F.y, a.y), fmaf(pc.selfVF, F.z, a.z)};
 #pragma unroll
   for (int c = 0; c < 3; ++c) U[o + c] = ADD ? U[o + c] + u[c] : u[c];
   if (W) {
-    const float4 b = psum[2 * s + 1], T = cT[s];
+    const float4 T = cT[s];
     const float w[3] = {fmaf(pc.selfWT, T.x, b.x), fmaf(pc.selfWT, T.y, b.y), fmaf(pc.selfWT, T.z, b.z)};
 #pragma unroll
     for (int c = 0; c < 3; ++c) W[o + c] = ADD ? W[o + c] + w[c] : w[c];
@@ -463,12 +516,14 @@ static void cluster_variant(const Geometry<float>& g, const PairConsts<float>& p
   const size_t smem = cluster_smem<TORQUE, WARPS>();
   auto k = pair_cluster_kernel<TORQUE, SHIFT, WARPS>;
   allow_dynamic_smem(k, smem);
-  k<<<b.ncells, WARPS * 32, smem, s>>>(g, pc, tab, poly, (const float4*)b.c_pos, (const float4*)b.c_F,
-                                       (const float4*)b.c_T, b.cell_start, (float4*)b.c_sum);
+  const int sharers = cell_blocks(WARPS, TORQUE) * device_sm_count();
+  k<<<std::max(b.ncells, sharers), WARPS * 32, smem, s>>>(g, pc, tab, poly, (const float4*)b.c_pos, (const float4*)b.c_F,
+                                       (const float4*)b.c_T, b.cell_start, (float4*)b.c_sum, b.c_sum64,
+                                     b.crowd, b.ncells, sharers);
 }
 
 // Warps of a CTA: a cell's clusters are dealt out to them, so cells of about eight particles (two clusters; the cell
-// size rule aims at eight) take two and fuller ones four. Measured with 2 / 4 / 8 warps: 122,231 particles in cells
+// size rule aims at eight) take two and fuller ones four; crowded cells are shared out in either. Measured with 2 / 4 / 8 warps: 122,231 particles in cells
 // of 8.8, forces only, 95 / 141 / 268 us; rods at 8.2 per cell, torques, 0.69 / 0.77 / 1.38 ms; 32 systems at 38 per
 // cell 3.14 / 2.87 / 3.47 ms; rigid rods, 12 per cell on average but all in one layer of three, 73 / 55 / 63 us.
 constexpr double kTwoWarpCell = 10.0;
@@ -497,8 +552,8 @@ void launch_pair_merge(const PairConsts<float>& pc, bool torque, const BinBuffer
                        cudaStream_t s, long long* launches) {
   if (n <= 0) return;
   auto k = add ? pair_merge_kernel<true> : pair_merge_kernel<false>;
-  k<<<(n + 255) / 256, 256, 0, s>>>(pc, (const float4*)b.c_sum, (const float4*)b.c_F, (const float4*)b.c_T, b.cell_rank,
-                                    n, b.n_dev, U, torque ? W : nullptr);
+  k<<<(n + 255) / 256, 256, 0, s>>>(pc, (const float4*)b.c_sum, b.c_sum64, b.crowd, (const float4*)b.c_F,
+                                    (const float4*)b.c_T, b.cell_rank, n, b.n_dev, U, torque ? W : nullptr);
   *launches += 1;
 }
 

@@ -41,9 +41,11 @@ constexpr size_t kCells = FCM_NOALLOC_MAX_CELLS;
 constexpr size_t kKeysBytes = align_up(2 * sizeof(unsigned) * kN);
 constexpr size_t kCellCountBytes = align_up(2 * sizeof(int) * (kCells + 4));
 constexpr size_t kSortedBytes = align_up(5 * sizeof(float4) * kN);
+constexpr size_t kSum64Bytes = align_up(6 * sizeof(double) * kN);
+constexpr size_t kCrowdBytes = align_up(sizeof(int) * crowd_ints(kN));
 constexpr size_t kTableBytes = align_up(5 * sizeof(float4) * kPairTableIntervals);
 constexpr size_t kStatusBytes = kAlign;
-constexpr size_t kScratchBytes = kKeysBytes + kCellCountBytes + kSortedBytes + kTableBytes + kStatusBytes;
+constexpr size_t kScratchBytes = kKeysBytes + kCellCountBytes + kSortedBytes + kSum64Bytes + kCrowdBytes + kTableBytes + kStatusBytes;
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -157,6 +159,10 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
   b.c_F = sorted + 3 * kN;
   b.c_T = sorted + 4 * kN;
   q += kSortedBytes;
+  b.c_sum64 = (double*)q;
+  q += kSum64Bytes;
+  b.crowd = (int*)q;
+  q += kCrowdBytes;
   float4* table = (float4*)q;
   q += kTableBytes;
   b.status = (int*)q;
