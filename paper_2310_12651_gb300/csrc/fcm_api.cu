@@ -305,19 +305,22 @@ static bool fit_pair_poly_from(const PairConsts<double>& pd, double a, double rn
 }
 
 // The smallest r_near on a ladder from 3 sigma to 0.6 r_c (past it too many pairs would be near ones) whose fit holds
-// (the error falls with r_near). The last result of the thread is kept, since callers without a handle ask for the
-// same parameters call after call.
+// (the error falls with r_near). A fit takes 0.2 to 0.5 ms of the host, and callers without a handle ask for the same few
+// parameter sets call after call, so each thread keeps its last eight.
 void fit_pair_poly(const PairConsts<double>& pd, double a, double r_c, PairPoly* out) {
-  struct Last {
+  struct Fit {
     double key[6];
     PairPoly poly;
   };
-  thread_local Last last{};
+  constexpr int kFits = 8;
+  thread_local Fit fits_kept[kFits] = {};
+  thread_local int oldest = 0;
   const double key[6] = {a, pd.eta, pd.Sg2, pd.SD2, r_c, pd.sg2};
-  if (std::memcmp(key, last.key, sizeof(key)) == 0 && r_c > 0.0) {
-    *out = last.poly;
-    return;
-  }
+  for (const Fit& f : fits_kept)
+    if (std::memcmp(key, f.key, sizeof(key)) == 0 && r_c > 0.0) {
+      *out = f.poly;
+      return;
+    }
   PairPoly best;
   std::memset(&best, 0, sizeof(best));
   const double r0 = 3.0 * std::sqrt(pd.sg2), step = 1.12;
@@ -338,8 +341,9 @@ void fit_pair_poly(const PairConsts<double>& pd, double a, double r_c, PairPoly*
       while (k < top && !fits(k + 1)) ++k;
     }
   }
-  std::memcpy(last.key, key, sizeof(key));
-  last.poly = best;
+  std::memcpy(fits_kept[oldest].key, key, sizeof(key));
+  fits_kept[oldest].poly = best;
+  oldest = (oldest + 1) % kFits;
   *out = best;
 }
 
