@@ -7,9 +7,9 @@
 // start offsets used by the pair correction. The rank of a particle inside its
 // bin is the value its atomic increment returned, so three kernels suffice:
 // key+count, scan, scatter. The scatter leaves the counters at zero for the next call.
-// Inside an 8-point tile particles are ordered by the quarter of the tile's x range their
-// window starts in (four counters per tile, one scan over them all): the pencil spreads
-// step along x in parts of a tile.
+// Inside an 8-point tile particles are ordered by the half of the tile's x range their
+// window starts in (two counters per tile, one scan over them all): the pencil spread
+// steps along x by half a tile.
 #include "fcm_internal.cuh"
 
 namespace fcm {
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, co
     }
     unsigned tk = (unsigned)(t[0] + g.ntile[0] * (t[1] + g.ntile[1] * t[2]));
     if (sys) tk += (unsigned)sys * (unsigned)g.tiles_per;
-    tk = kTileParts * tk + (g.tile[0] == 2 * kTileParts ? (unsigned)(xoff >> 1) : 0u);
+    tk = kTileParts * tk + (g.tile[0] == 8 ? (unsigned)(xoff / (8 / kTileParts)) : 0u);
     b.tile_key[i] = tk;
     b.tile_rank[i] = (unsigned)atomicAdd(&b.tile_count[tk], 1);
   }
@@ -201,8 +201,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
                                                       BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   // the counters back to zero for the next call (16 bytes per store; the arrays are padded to 256 bytes)
-  const int nz_t = (need & kBinTiles) ? b.ntiles : 0, nz_c = (need & kBinCells) ? (b.cell_parts * b.ncells + 3) / 4 : 0;
-  static_assert(kTileParts == 4, "one 16-byte store per tile");
+  const int nz_t = (need & kBinTiles) ? (kTileParts * b.ntiles + 3) / 4 : 0, nz_c = (need & kBinCells) ? (b.cell_parts * b.ncells + 3) / 4 : 0;
   for (int k = i; k < nz_t + nz_c; k += gridDim.x * blockDim.x)
     (k < nz_t ? reinterpret_cast<int4*>(b.tile_count)[k] : reinterpret_cast<int4*>(b.cell_count)[k - nz_t]) =
         make_int4(0, 0, 0, 0);
@@ -264,7 +263,7 @@ void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const
   }
   scan_kernel<<<grid, kScanThreads, 0, s>>>(b, tile_chunks, sums ? 1 : 0);
   // enough blocks for the particles and for at most eight counter stores per thread
-  const int zero_blocks = (int)(((long long)tiles + cells / 4 + 1 + 2047) / 2048);
+  const int zero_blocks = (int)((((long long)kTileParts * tiles + cells) / 4 + 2 + 2047) / 2048);
   scatter_kernel<R><<<std::max(blocks, zero_blocks), 256, 0, s>>>(g, n, pos, F, T, b, need);
   *launches += 2;
 }

@@ -282,7 +282,7 @@ void narrow_pair_consts(const PairConsts<double>& in, PairConsts<float>* out);
 void build_pair_table(const PairConsts<double>& pd, double r_lo, double r_hi, int n, float4* coef);
 
 // ---------------------------------------------------------------- launch API
-constexpr int kTileParts = 4;       // parts of an 8-point tile's x range by which its particles are ordered
+constexpr int kTileParts = 2;       // parts of an 8-point tile's x range by which its particles are ordered
 constexpr int kScanThreads = 512;
 constexpr int kScanChunk = 2048;    // counters per block of the scan
 inline int scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
