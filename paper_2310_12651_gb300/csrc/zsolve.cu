@@ -35,7 +35,7 @@ template <> struct Pair2<double> { typedef double2 T; };
 __device__ inline int quot(int n, unsigned magic) { return magic ? (int)__umulhi((unsigned)n, magic) : n; }
 
 template <typename R>
-struct C {
+struct alignas(2 * sizeof(R)) C {   // as the float2 or double2 it is read as
   R x, y;
 };
 template <typename R> __device__ inline C<R> operator+(C<R> a, C<R> b) { return {a.x + b.x, a.y + b.y}; }
