@@ -5,7 +5,8 @@
 // and shared-memory work beside them is free. The kernel's polynomial P = A + B (dx^2 + dy^2 + dz^2) and
 // the torque's cross products are split into one-dimensional tables and per-row coefficients.
 //
-// * spread: f_c(x) += G alpha_c g(x) + G w_c(x), two FMAs per point and component (Sigma_D = Sigma);
+// * spread: f_c(x) += G alpha_c g(x) + G w_c(x), two FMAs per point and component (Sigma_D = Sigma; two widths take
+//   five more per point, from the torque's own row factors);
 //   threads take window points in x-fastest order, so the FP64 reductions of a row are contiguous;
 // * gather: a thread per window row, eight FMAs per point (the x moments of u), then the row's factors;
 //   the six sums are reduced across lanes by halving the values with the lanes (nine additions, not 30).
@@ -60,7 +61,9 @@ __global__ void __launch_bounds__(kSpread64Threads) spread_bpp_f64(Geometry<doub
   __shared__ double wx[3][kMaxMG];     // B F'_c d^2 g (+ the torque's d g) along x
   __shared__ double ay[3][kMaxMG], az[3][kMaxMG];   // alpha_c split into its y and z parts
   __shared__ Vec4<double> row[kMaxRows];   // {G alpha_x, G alpha_y, G alpha_z, G}
-  __shared__ double hrow[SAMEW || !TORQUE ? 1 : kMaxRows];   // two widths: tq g_D(dy) g_D(dz)
+  constexpr bool TWO = TORQUE && !SAMEW;   // the torque has a Gaussian of its own, H = g_D(dy) g_D(dz)
+  __shared__ Vec4<double> trow[TWO ? kMaxRows : 1];   // H {U'y dz - U'z dy, -U'x dz, U'x dy, 1}
+  __shared__ double tx[2][TWO ? kMaxMG : 1];          // U'z d g_D and -U'y d g_D along x
   __shared__ long long off[kMaxRows];
   const int p = blockIdx.x;
   const Vec4<double> y = pos[p];
@@ -77,6 +80,10 @@ __global__ void __launch_bounds__(kSpread64Threads) spread_bpp_f64(Geometry<doub
     const int d = k / MG, j = k - d * MG;
     const double dd = t.d[d][j], bq = kc.B * dd * dd;
     if (d == 0) {
+      if (TWO) {
+        tx[0][j] = Uz * dd * t.gd[0][j];
+        tx[1][j] = -Uy * dd * t.gd[0][j];
+      }
       const double q = bq * t.g[0][j], dg = dd * t.g[0][j];
       wx[0][j] = Fx * q;
       wx[1][j] = FOLD ? fma(Uz, dg, Fy * q) : Fy * q;
@@ -97,7 +104,10 @@ __global__ void __launch_bounds__(kSpread64Threads) spread_bpp_f64(Geometry<doub
     const int jz = r / MG, jy = r - jz * MG;
     const double G = t.g[1][jy] * t.g[2][jz];
     row[r] = {G * (ay[0][jy] + az[0][jz]), G * (ay[1][jy] + az[1][jz]), G * (ay[2][jy] + az[2][jz]), G};
-    if (TORQUE && !SAMEW) hrow[r] = t.gd[1][jy] * t.gd[2][jz];
+    if (TWO) {
+      const double H = t.gd[1][jy] * t.gd[2][jz], dy = t.d[1][jy], dz = t.d[2][jz];
+      trow[r] = {H * fma(Uy, dz, -Uz * dy), -H * Ux * dz, H * Ux * dy, H};
+    }
     off[r] = ((long long)at[2][jz] * g.M[1] + at[1][jy]) * g.M[0];
   }
   __syncthreads();
@@ -111,13 +121,12 @@ __global__ void __launch_bounds__(kSpread64Threads) spread_bpp_f64(Geometry<doub
     double fx = fma(a.w, wx[0][j], a.x * gx);
     double fy = fma(a.w, wx[1][j], a.y * gx);
     double fz = fma(a.w, wx[2][j], a.z * gx);
-    if (TORQUE && !SAMEW) {
-      const int jz = r / MG, jy = r - jz * MG;
-      const double wt = hrow[r] * t.gd[0][j];
-      const double dx = t.d[0][j], dy = t.d[1][jy], dz = t.d[2][jz];
-      fx = fma(wt, fma(Uy, dz, -Uz * dy), fx);
-      fy = fma(wt, fma(Uz, dx, -Ux * dz), fy);
-      fz = fma(wt, fma(Ux, dy, -Uy * dx), fz);
+    if (TWO) {
+      const Vec4<double> c = trow[r];
+      const double gd = t.gd[0][j];
+      fx = fma(c.x, gd, fx);
+      fy = fma(c.y, gd, fma(c.w, tx[0][j], fy));
+      fz = fma(c.z, gd, fma(c.w, tx[1][j], fz));
     }
     double* q = grid + off[r] + at[0][j];
     atomicAdd(q, fx);
