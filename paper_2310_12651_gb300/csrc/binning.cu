@@ -29,7 +29,7 @@ template <typename R>
 __global__ void __launch_bounds__(256) key_count_kernel(Geometry<R> g, int n, const R* __restrict__ pos,
                                                         BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && (need & kBinCells) && b.crowd) b.crowd[1] = 0;   // for the scan to fill
+  if (i == 0 && (need & kBinCells)) b.crowd[1] = 0;   // for the scan to fill
   if (b.n_dev) n = min(n, *b.n_dev);
   if (i >= n) return;
   const int sys = system_of(b, i);
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(BinBuffers b, int ti
     v[k] = first + k < p.nb ? p.count[first + k] : 0;
     own += v[k];
   }
-  if (!p.tiles && b.crowd) {
+  if (!p.tiles) {
     const int at = (int)blockIdx.y * p.nb + first;   // the thread's first counter
     static_assert(kPer == 4, "two neighbouring threads per cell of eight counters");
     if (b.cell_parts == 8) {

@@ -846,7 +846,7 @@ size_t workspace_estimate(const fcm_params& p, int max_systems) {
   const size_t mtot = (size_t)p.M[0] * p.M[1] * p.M[2];
   const size_t ncplx = (size_t)(p.M[0] / 2 + 1) * p.M[1] * p.M[2];
   const size_t ntiles = (size_t)g.tiles_per * gsys, ncells = (size_t)g.cells_per * gsys;
-  size_t b = 16 * n + 4 * ((2 * kTileParts + 1) * ntiles + 2) + 4 * ((fp64 ? 1 : 17) * ncells + 2) + 4 * (ncells + 1) + (kTileParts * ntiles + 8 * ncells) / 512 + 8 * gsys + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + (fp64 ? 9 * rsz * n : 23 * rsz * n + sizeof(int) * crowd_ints(n));
+  size_t b = 16 * n + 4 * ((2 * kTileParts + 1) * ntiles + 2) + 4 * ((fp64 ? 1 : 17) * ncells + 2) + 4 * (ncells + 1) + (kTileParts * ntiles + 8 * ncells) / 512 + 8 * gsys + 6 * v4 * n + 256 + 4 * (kMaxBatch + 1) + (fp64 ? 9 : 23) * rsz * n + sizeof(int) * crowd_ints(n);
   size_t table = sizeof(float4) * 5 * kPairTableIntervals;
   if (fp64) {
     const double r_lo = 0.5 * p.a / std::sqrt(kPi);   // (r_c may be anything where no pairs act: bounded by the box)
@@ -1459,10 +1459,9 @@ int fcm_create_batch(const fcm_params* p, int max_systems, int device, fcm_handl
     work = std::max(work, std::max(w1, w2));
   }
   A(&h->fft_work, work);
-  if (!h->fp64) {   // after the grids: the transforms' time depends on where those lie
-    A((void**)&b.c_sum64, 6 * sizeof(double) * n);
-    A((void**)&b.crowd, sizeof(int) * crowd_ints(n));
-  }
+  // after the grids: the transforms' time depends on where those lie
+  if (!h->fp64) A((void**)&b.c_sum64, 6 * sizeof(double) * n);
+  A((void**)&b.crowd, sizeof(int) * crowd_ints(n));
   if (rc != FCM_OK) { std::string e = g_error; release(h); return fail(rc, e); }
   for (auto& pl : h->plans) {
     if (cufftSetWorkArea(pl.r2c, h->fft_work) != CUFFT_SUCCESS || cufftSetWorkArea(pl.c2r, h->fft_work) != CUFFT_SUCCESS) {

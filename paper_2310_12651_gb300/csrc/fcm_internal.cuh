@@ -287,8 +287,8 @@ constexpr int kScanThreads = 512;
 constexpr int kScanChunk = 2048;    // counters per block of the scan
 inline int scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
 enum : int { kBinTiles = 1, kBinCells = 2 };   // which of the two orders a call needs
-// FP32 pair cells of more than kCrowdCell particles are crowded: their clusters are shared out in parts of about
-// kCrowdPart particles and their sums are in FP64 (pair_f32.cu). Every such cell of n makes ceil(n / kCrowdPart) items.
+// Pair cells of more than kCrowdCell particles are crowded: they are shared out in parts of about kCrowdPart particles and
+// their sums are in FP64 also in FP32 (pair_f32.cu, pair_f64.cu). A cell of n makes ceil(n / kCrowdPart) items.
 constexpr int kCrowdCell = 96, kCrowdPart = 32;
 __host__ __device__ inline int crowd_parts(int n) { return (n + kCrowdPart - 1) / kCrowdPart; }
 constexpr size_t crowd_ints(size_t n) { return 2 + 2 * (n / (kCrowdCell / 4) + 1); }   // 97 particles make four items
@@ -310,7 +310,7 @@ struct BinBuffers {
   void* c_pos; void* c_F; void* c_T;   // cell-sorted Vec4<R>
   void* c_sum;   // FP32: pair sums (float4 of U, float4 of W) per cell-sorted particle, cleared by the scatter
   double* c_sum64;   // FP32: those from crowded cells (three of U, three of W), cleared where there is such a cell
-  int* crowd;    // FP32 (else null): items of crowded cells, written by the scan: [1] how many, from [2] on cell and part
+  int* crowd;    // items of crowded cells, written by the scan: [1] how many, from [2] on cell and part
   int* status;
   // Batched launches: particles of system s are rows sys_off[s] .. sys_off[s+1]-1 of the stacked
   // inputs (device array of nsys + 1 ints); nsys <= 1 or sys_off == nullptr is one system.

@@ -150,22 +150,19 @@ __device__ __forceinline__ void eval_pair64(const Geometry<double>& g, const Pai
   }
 }
 
-// CTA (cell, part): the particles i of the cell with (i - first) mod gridDim.y == part, against the half shell.
+// The particles i of the cell with (i - first) mod parts == part, against the half shell.
 template <bool TORQUE>
-__global__ void __launch_bounds__(kWarps64 * 32) pair_half_f64(Geometry<double> g, PairConsts<double> pc,
-                                                               PairTable64 tab, double inv, float rc2f,
-                                                               const Vec4<double>* __restrict__ cpos,
-                                                               const Vec4<double>* __restrict__ cF,
-                                                               const Vec4<double>* __restrict__ cT,
-                                                               const int* __restrict__ cstart,
-                                                               double* __restrict__ Uo, double* __restrict__ Wo) {
+__device__ __forceinline__ void half_cell64(const Geometry<double>& g, const PairConsts<double>& pc,
+                                            const PairTable64& tab, double inv, float rc2f,
+                                            const Vec4<double>* __restrict__ cpos, const Vec4<double>* __restrict__ cF,
+                                            const Vec4<double>* __restrict__ cT, const int* __restrict__ cstart,
+                                            double* __restrict__ Uo, double* __restrict__ Wo, int cell, int part,
+                                            int parts) {
   __shared__ float4 spos[kChunk64];       // x, y, z over the longest box edge in FP32, cell-sorted index
   __shared__ int2 queue[kWarps64][kQueue64];
   __shared__ int meta[2 * kPieces + 2];
   __shared__ float4 shift[kPieces];
-  const int cell = blockIdx.x;
   const int i_begin = cstart[cell], i_end = cstart[cell + 1];
-  if (i_begin + (int)blockIdx.y >= i_end) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp == 0) half_shell_pieces(g, cell, cstart, meta, shift);
   __syncthreads();
@@ -186,7 +183,7 @@ __global__ void __launch_bounds__(kWarps64 * 32) pair_half_f64(Geometry<double> 
       }
     }
     __syncthreads();
-    for (int i = i_begin + blockIdx.y + gridDim.y * warp; i < i_end; i += gridDim.y * kWarps64) {
+    for (int i = i_begin + part + parts * warp; i < i_end; i += parts * kWarps64) {
       const Vec4<double> yd = cpos[i];
       const float yx = (float)(yd.x * inv), yy = (float)(yd.y * inv), yz = (float)(yd.z * inv);
       if (cb == 0 && lane < 3) {   // the self terms of Appendix B
@@ -235,6 +232,40 @@ __global__ void __launch_bounds__(kWarps64 * 32) pair_half_f64(Geometry<double> 
   }
 }
 
+// CTA b takes part b mod `parts` of cell b / parts, unless the cell is crowded. The last `sharers` CTAs then share the
+// crowded cells' parts, which the binning's scan lists (kSplit64 CTAs to a listed part): 20,000 particles in one cell of
+// many would otherwise run in one CTA (1,329 ms; a thread per particle over 27 cells, the kernel before this one, 942 ms;
+// so 8.2 ms).
+constexpr int kSplit64 = 4;
+
+template <bool TORQUE>
+__global__ void __launch_bounds__(kWarps64 * 32) pair_half_f64(Geometry<double> g, PairConsts<double> pc,
+                                                               PairTable64 tab, double inv, float rc2f,
+                                                               const Vec4<double>* __restrict__ cpos,
+                                                               const Vec4<double>* __restrict__ cF,
+                                                               const Vec4<double>* __restrict__ cT,
+                                                               const int* __restrict__ cstart,
+                                                               double* __restrict__ Uo, double* __restrict__ Wo,
+                                                               const int* __restrict__ crowd, int ncells, int nparts,
+                                                               int sharers) {
+  int cell = blockIdx.x / nparts, part = blockIdx.x - cell * nparts, parts = nparts;
+  const int place = (int)blockIdx.x - ((int)gridDim.x - sharers);   // among the sharers
+  bool own = cell < ncells;   // first the CTA's own cell, then every sharers-th item
+  for (int k = own ? place - sharers : place;; k += sharers) {
+    if (!own) {
+      if (k < 0 || k >= kSplit64 * crowd[1]) return;
+      cell = crowd[2 + 2 * (k / kSplit64)];
+      part = kSplit64 * crowd[3 + 2 * (k / kSplit64)] + k % kSplit64;
+    }
+    const int n = cstart[cell + 1] - cstart[cell];
+    if (!own) parts = kSplit64 * crowd_parts(n);
+    if (part < n && (!own || n <= kCrowdCell))
+      half_cell64<TORQUE>(g, pc, tab, inv, rc2f, cpos, cF, cT, cstart, Uo, Wo, cell, part, parts);
+    own = false;
+    __syncthreads();   // the next part reuses the shared memory
+  }
+}
+
 }  // namespace
 
 void pair_table64_range(double rs2, double rc2, int* base, int* n) {
@@ -264,14 +295,16 @@ void launch_pair_f64(const Geometry<double>& g, const PairConsts<double>& pc, co
   const float rc2f = (float)(reach * reach * (1.0 + 1e-5));
   // parts of a cell: enough CTAs for four per SM when the cells are few
   const int parts = std::min(16, std::max(1, (4 * device_sm_count() + b.ncells - 1) / b.ncells));
-  const dim3 grid(b.ncells, parts);
+  const int sharers = 4 * device_sm_count(), grid = std::max(b.ncells * parts, sharers);
   const Vec4<double>* pos = (const Vec4<double>*)b.c_pos;
   const Vec4<double>* F = (const Vec4<double>*)b.c_F;
   const Vec4<double>* T = (const Vec4<double>*)b.c_T;
   if (torque)
-    pair_half_f64<true><<<grid, kWarps64 * 32, 0, s>>>(g, pc, tab, 1.0 / Lmax, rc2f, pos, F, T, b.cell_start, upair, wpair);
+    pair_half_f64<true><<<grid, kWarps64 * 32, 0, s>>>(g, pc, tab, 1.0 / Lmax, rc2f, pos, F, T, b.cell_start,
+                                                            upair, wpair, b.crowd, b.ncells, parts, sharers);
   else
-    pair_half_f64<false><<<grid, kWarps64 * 32, 0, s>>>(g, pc, tab, 1.0 / Lmax, rc2f, pos, F, T, b.cell_start, upair, wpair);
+    pair_half_f64<false><<<grid, kWarps64 * 32, 0, s>>>(g, pc, tab, 1.0 / Lmax, rc2f, pos, F, T, b.cell_start,
+                                                            upair, wpair, b.crowd, b.ncells, parts, sharers);
   *launches += 1;
 }
 

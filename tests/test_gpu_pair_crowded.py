@@ -1,9 +1,10 @@
-"""The FP32 pair kernel's crowded cells (more than 96 particles): their parts are shared out and summed in FP64, in
-launches of two and of four warps per cell, beside cells that are not crowded, and none is left from an earlier call."""
+"""The pair kernels' crowded cells (more than 96 particles): their parts are shared out and summed in FP64, in FP32
+in launches of two and of four warps per cell, beside cells that are not crowded, and none is left from an earlier call."""
 import numpy as np
 import pytest
 
-from gpu_util import System, ensure_built, params_for, rel_l2, rounded, run_gpu, torch_cuda
+from gpu_util import (FP64_TOL, System, assert_parity, ensure_built, params_for, rel_l2, rounded, run_gpu,
+                      torch_cuda)
 
 pytestmark = pytest.mark.gpu
 
@@ -105,3 +106,22 @@ def test_crowded_cells_without_allocation():
                                     torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert rel_l2(U.double().cpu().numpy(), U64) < BAR and rel_l2(W.double().cpu().numpy(), W64) < BAR
+
+
+@pytest.mark.parametrize("n,L,corner,r_c,torques", [
+    (1500, 100.0, 19.9, 9.9, True),     # one cell of 1,500
+    (1500, 100.0, 19.9, 9.9, False),
+    (3000, 34.0, 34.0, 11.3, True),     # every cell crowded
+    (700, 100.0, 24.0, 9.9, True),      # crowded cells among empty and ordinary ones
+])
+def test_crowded_cells_fp64(n, L, corner, r_c, torques):
+    """The same sharing out in FP64, against the oracle."""
+    fcm = ensure_built()
+    s = System(n, L, 32, 1.6, 8, r_c, 3, torques=torques, Y=_corner(n, L, corner, n))
+    count, _ = _cells(s, n)
+    assert count.max() > CROWD
+    U, W = run_gpu(s, fcm.FCM_FP64, stages=2, want_W=torques)
+    Uo, Wo = s.oracle(fcm.FCM_FP64, stages=2)
+    assert_parity(U, Uo, FP64_TOL, "U")
+    if torques:
+        assert_parity(W, Wo, FP64_TOL, "W")
