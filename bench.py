@@ -1273,7 +1273,7 @@ def main():
         stages_out["fft_solve"]["ms_alone"] = fft_alone
         stages_out["fft_solve"]["GBps"] = fft_bytes / (fft_alone * 1e-3) / 1e9
         stages_out["fft_solve"]["frac_hbm"] = stages_out["fft_solve"]["GBps"] / hbm
-        stages_out["fft_solve"]["bytes"] = "72 B per grid point: 6 transforms x 8 B + 24 B for the projection kernel"
+        stages_out["fft_solve"]["bytes"] = "72 B per grid point, 24 B read and written by each of the (x, y) transforms, the z transforms with the operator, and the (x, y) transforms back"
     if gather_alone:
         stages_out["gather"]["ms_alone"] = gather_alone
     if pair_alone:

@@ -57,7 +57,8 @@ typedef enum fcm_precision {
   FCM_FP32 = 0,  /* float I/O; tiled spread/gather, FP32 FFT; pair corrections from  */
                  /* polynomials in 1/r times a Gaussian beyond a few particle radii   */
                  /* and piecewise cubics closer, both fitted in FP64 to the closed     */
-                 /* forms, and a Taylor series below sigma/2                           */
+                 /* forms, and a Taylor series below sigma/2; pair sums in FP32, in    */
+                 /* pair cells of more than 96 particles in FP64 (order not fixed)     */
   FCM_FP64 = 1   /* double I/O; the plain path: global FP64 atomics, FP64 FFT        */
 } fcm_precision;
 

@@ -6,7 +6,8 @@
 // tile-sorted arrays used by spread/gather and the cell-sorted arrays with
 // start offsets used by the pair correction. The rank of a particle inside its
 // bin is the value its atomic increment returned, so three kernels suffice:
-// key+count, scan, scatter. The scatter leaves the counters at zero for the next call.
+// key+count, scan, scatter (and a fourth that adds up chunks of counters, where the
+// scan has many). The scatter leaves the counters at zero for the next call.
 // Inside an 8-point tile particles are ordered by the half of the tile's x range their
 // window starts in (two counters per tile, one scan over them all): the pencil spread
 // steps along x by half a tile.
@@ -255,7 +256,7 @@ void launch_binning(const Geometry<R>& g, int n, const R* pos, const R* F, const
   if (need == 0) return;   // no order needed (a correction that is identically zero): the position check alone
   // Every block reading all counters before its chunk costs chunks^2 / 2 chunk reads from L2: below a microsecond
   // at 16 chunks, 8 at 64 (each block's own reads are a chain of loads); past that the chunk sums pay their launch.
-  const bool sums = std::max(tile_chunks, cell_chunks) > 32 && b.chunk_sum != nullptr;
+  const bool sums = std::max(tile_chunks, cell_chunks) > kScanSumsAbove && b.chunk_sum != nullptr;
   const dim3 grid(tile_chunks + cell_chunks, nsys);
   if (sums) {
     chunk_sum_kernel<<<grid, kScanThreads, 0, s>>>(b, tile_chunks);

@@ -285,7 +285,8 @@ void build_pair_table(const PairConsts<double>& pd, double r_lo, double r_hi, in
 constexpr int kTileParts = 2;       // parts of an 8-point tile's x range by which its particles are ordered
 constexpr int kScanThreads = 512;
 constexpr int kScanChunk = 2048;    // counters per block of the scan
-inline int scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
+constexpr int kScanSumsAbove = 32;  // chunks above which the scan starts from their sums
+constexpr int scan_chunks(int n) { return (n + kScanChunk - 1) / kScanChunk; }
 enum : int { kBinTiles = 1, kBinCells = 2 };   // which of the two orders a call needs
 // Pair cells of more than kCrowdCell particles are crowded: they are shared out in parts of about kCrowdPart particles and
 // their sums are in FP64 also in FP32 (pair_f32.cu, pair_f64.cu). A cell of n makes ceil(n / kCrowdPart) items.
@@ -304,7 +305,7 @@ struct BinBuffers {
   int* cell_count;    // cell_parts counters per cell: its octants along a path of neighbours (8), or the cell (1)
   int* cell_part_start;   // first particle of every part (cell_start itself where cell_parts == 1)
   int* cell_start; int cell_parts;
-  int* chunk_sum;     // scan: sums of kScanChunk counters (may be null for few chunks)
+  int* chunk_sum;     // scan: sums of kScanChunk counters (null where chunks are never more than kScanSumsAbove)
   int ntiles; int ncells;
   void* t_pos; void* t_F; void* t_T;   // tile-sorted Vec4<R>
   void* c_pos; void* c_F; void* c_T;   // cell-sorted Vec4<R>

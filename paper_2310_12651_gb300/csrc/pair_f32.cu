@@ -35,8 +35,9 @@
 //   neighbours 245 / 282 / 216, 4,000 in one cell 149 / 203 / 146. Sharing out keeps a suspension that fills a corner
 //   of its box from running in a few CTAs: 65,536 in 125 cells 2.76 / 3.58 / 0.69 ms, 4,000 in one cell 11.9 / 9.3 / 0.21 ms.
 // Measured against one particle at a time, tables and shared-memory atomics: 32 systems of 65,536 at 5%, torques,
-// 4.04 -> 2.93 ms; 1,048,576 at 10% 2.64 -> 1.84 ms; 122,231 at 0.8%, forces only, 153 -> 95 us. Now 1,020
-// instructions per particle, the schedulers issue 58% of the time and the FMA pipe is busy 45%.
+// 4.04 -> 2.82 ms; 1,048,576 at 10% 2.64 -> 1.77 ms; 122,231 at 0.8%, forces only, 153 -> 100 us; without a fit (Sigma_D =
+// 1.27 Sigma, every pair by the table) 65,536 at 5% 122 -> 117 us. Now 1,023 instructions per particle, the schedulers
+// issue 59% of the time and the FMA pipe is busy 46%.
 #include "pair_common.cuh"
 
 namespace fcm {

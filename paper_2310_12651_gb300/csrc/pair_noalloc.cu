@@ -38,6 +38,7 @@ constexpr size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign;
 
 constexpr size_t kN = FCM_NOALLOC_MAX_N;
 constexpr size_t kCells = FCM_NOALLOC_MAX_CELLS;
+static_assert(scan_chunks(FCM_NOALLOC_MAX_CELLS) <= kScanSumsAbove, "the scan of the cells has no room for chunk sums here");
 constexpr size_t kKeysBytes = align_up(2 * sizeof(unsigned) * kN);
 constexpr size_t kCellCountBytes = align_up(2 * sizeof(int) * (kCells + 4));
 constexpr size_t kSortedBytes = align_up(5 * sizeof(float4) * kN);
@@ -183,7 +184,7 @@ extern "C" int fcm_pair_correction_noalloc(const fcm_params* p, int n, const voi
 
   cudaStream_t s = (cudaStream_t)stream;
   long long launches = 0;
-  // counters must start at zero; the scan leaves them at zero, but a call may follow an error
+  // counters must start at zero; the scatter leaves them at zero, but a call may follow an error
   launch_zero(b.cell_count, sizeof(int) * (size_t)(cells + 1), s, &launches);
   launch_zero(b.status, kStatusBytes, s, &launches);
   build_table_kernel<<<(kPairTableIntervals + 127) / 128, 128, 0, s>>>(pd, r_lo, (r_hi - r_lo) / kPairTableIntervals,

@@ -7,11 +7,13 @@
 // takes neighbouring columns (contiguous in memory) of all three components, keeps them in
 // shared memory from the first read to the last write, and transforms them there: Stockham steps of radix 2
 // to 16 between two copies of the columns, the first reading and the last writing global memory.
-// Twiddle factors come from a table rounded from FP64. What bounds it in FP32 is HBM (16 bytes per
-// value) together with about 100 bytes per value of shared-memory traffic, which is the same time.
-// Measured against transforms and operator in three kernels: 32 systems of 128^3 841 -> 615 us, 256^3 261 -> 210 us,
-// 240 x 240 x 16 13.5 -> 9.2 us, 13 systems of 90 x 72 x 54 65 -> 49 us, FP64 64^3 80 -> 43 us. In FP32 the schedulers
-// issue half of the time (about 150 instructions per value, addresses and factors among them).
+// Twiddle factors come from a table rounded from FP64. What bounds it in FP32 is issue: about 150 instructions per
+// value, addresses and factors among them; the schedulers issue 57% of the time and next wait for instructions (the
+// unrolled butterflies of both directions) and for the first loads, while shared memory is busy 47% and HBM moves
+// its 16 bytes per value at 0.40 of the copy rate. Measured against transforms and operator in three kernels: 32
+// systems of 128^3 841 -> 591 us (615 with complex values declared at the alignment of one real, two accesses for
+// one), 256^3 261 -> 210 us, 240 x 240 x 16 13.5 -> 9.2 us, 13 systems of 90 x 72 x 54 65 -> 49 us, FP64 64^3 80 -> 43 us.
+// Lengths of threes alone gain nothing (243^3: the whole chain 585 -> 611 us, 8 x 81^3 146 -> 147 us).
 #include <cmath>
 #include <vector>
 
