@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
                                                       const R* __restrict__ F, const R* __restrict__ T,
                                                       BinBuffers b, int need) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool crowded = (need & kBinCells) && b.crowd[1] > 0;
   // the counters back to zero for the next call (16 bytes per store; the arrays are padded to 256 bytes)
   const int nz_t = (need & kBinTiles) ? (kTileParts * b.ntiles + 3) / 4 : 0, nz_c = (need & kBinCells) ? (b.cell_parts * b.ncells + 3) / 4 : 0;
   for (int k = i; k < nz_t + nz_c; k += gridDim.x * blockDim.x)
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(Geometry<R> g, int n, cons
       const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
       ((float4*)b.c_sum)[2 * (size_t)dc] = zero;
       ((float4*)b.c_sum)[2 * (size_t)dc + 1] = zero;
-      if (b.crowd[1] > 0)
+      if (crowded)
         for (int k = 0; k < 3; ++k) reinterpret_cast<float4*>(b.c_sum64 + 6 * (size_t)dc)[k] = zero;
     }
     ((Vec4<R>*)b.c_pos)[dc] = p;

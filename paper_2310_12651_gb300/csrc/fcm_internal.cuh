@@ -292,7 +292,8 @@ enum : int { kBinTiles = 1, kBinCells = 2 };   // which of the two orders a call
 // their sums are in FP64 also in FP32 (pair_f32.cu, pair_f64.cu). A cell of n makes ceil(n / kCrowdPart) items.
 constexpr int kCrowdCell = 96, kCrowdPart = 32;
 __host__ __device__ inline int crowd_parts(int n) { return (n + kCrowdPart - 1) / kCrowdPart; }
-constexpr size_t crowd_ints(size_t n) { return 2 + 2 * (n / (kCrowdCell / 4) + 1); }   // 97 particles make four items
+constexpr int crowd_items(int n) { return n / (kCrowdCell / 4) + 1; }   // at most: 97 particles make four items
+constexpr size_t crowd_ints(size_t n) { return 2 + 2 * (size_t)crowd_items((int)n); }
 
 // Binning: wraps positions, computes tile and cell keys, counts and ranks,
 // scans, then scatters pos/F/T into tile-sorted and cell-sorted Vec4 arrays

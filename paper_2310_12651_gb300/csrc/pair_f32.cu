@@ -461,8 +461,8 @@ __device__ __forceinline__ void cell_pairs(const Geometry<float>& g, const PairC
   }
 }
 
-// CTA c takes cell c unless it is crowded. The last `sharers` CTAs (as many as run at once; more of them than cells where
-// cells are few) then share the crowded cells' parts.
+// CTA c takes cell c unless it is crowded. The last `sharers` CTAs (as many as run at once, at most one per possible part;
+// more of them than cells where cells are few) then share the crowded cells' parts.
 template <bool TORQUE, bool SHIFT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, cell_blocks(WARPS, TORQUE))
     pair_cluster_kernel(Geometry<float> g, PairConsts<float> pc, PairTable tab, PairPoly poly,
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256) pair_merge_kernel(PairConsts<float> pc, c
   if (i >= n) return;
   const size_t s = slot[i], o = 3 * (size_t)i;
   const float4 F = cF[s];
-  float4 a = psum[2 * s], b = psum[2 * s + 1];   // all loads before the branch
+  float4 a = psum[2 * s], b = W ? psum[2 * s + 1] : a;   // all loads before the branch
   if (crowd[1] > 0) {   // some sums are in FP64
     const double* q = psum64 + 6 * s;
     a = make_float4((float)(a.x + q[0]), (float)(a.y + q[1]), (float)(a.z + q[2]), 0.f);
@@ -513,11 +513,11 @@ __global__ void __launch_bounds__(256) pair_merge_kernel(PairConsts<float> pc, c
 
 template <bool TORQUE, bool SHIFT, int WARPS>
 static void cluster_variant(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab,
-                            const PairPoly& poly, const BinBuffers& b, cudaStream_t s) {
+                            const PairPoly& poly, const BinBuffers& b, int n, cudaStream_t s) {
   const size_t smem = cluster_smem<TORQUE, WARPS>();
   auto k = pair_cluster_kernel<TORQUE, SHIFT, WARPS>;
   allow_dynamic_smem(k, smem);
-  const int sharers = cell_blocks(WARPS, TORQUE) * device_sm_count();
+  const int sharers = std::min(cell_blocks(WARPS, TORQUE) * device_sm_count(), crowd_items(n));
   k<<<std::max(b.ncells, sharers), WARPS * 32, smem, s>>>(g, pc, tab, poly, (const float4*)b.c_pos, (const float4*)b.c_F,
                                        (const float4*)b.c_T, b.cell_start, (float4*)b.c_sum, b.c_sum64,
                                      b.crowd, b.ncells, sharers);
@@ -532,8 +532,8 @@ constexpr double kTwoWarpCell = 10.0;
 template <bool TORQUE, bool SHIFT>
 static void cluster_launch(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab,
                            const PairPoly& poly, const BinBuffers& b, int n, cudaStream_t s) {
-  if ((double)n < kTwoWarpCell * b.ncells) cluster_variant<TORQUE, SHIFT, 2>(g, pc, tab, poly, b, s);
-  else cluster_variant<TORQUE, SHIFT, 4>(g, pc, tab, poly, b, s);
+  if ((double)n < kTwoWarpCell * b.ncells) cluster_variant<TORQUE, SHIFT, 2>(g, pc, tab, poly, b, n, s);
+  else cluster_variant<TORQUE, SHIFT, 4>(g, pc, tab, poly, b, n, s);
 }
 
 void launch_pair_f32(const Geometry<float>& g, const PairConsts<float>& pc, const PairTable& tab, const PairPoly& poly,

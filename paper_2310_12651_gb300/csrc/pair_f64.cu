@@ -295,7 +295,7 @@ void launch_pair_f64(const Geometry<double>& g, const PairConsts<double>& pc, co
   const float rc2f = (float)(reach * reach * (1.0 + 1e-5));
   // parts of a cell: enough CTAs for four per SM when the cells are few
   const int parts = std::min(16, std::max(1, (4 * device_sm_count() + b.ncells - 1) / b.ncells));
-  const int sharers = 4 * device_sm_count(), grid = std::max(b.ncells * parts, sharers);
+  const int sharers = std::min(4 * device_sm_count(), kSplit64 * crowd_items(n)), grid = std::max(b.ncells * parts, sharers);
   const Vec4<double>* pos = (const Vec4<double>*)b.c_pos;
   const Vec4<double>* F = (const Vec4<double>*)b.c_F;
   const Vec4<double>* T = (const Vec4<double>*)b.c_T;
